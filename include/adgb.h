@@ -84,10 +84,13 @@ typedef struct {
     int pair_rounds;       /* intramolecular pairs: 0 = matching rounds (ligand_pair_rounds;
                               the default, faster at every size measured), 1 = per-pair
                               force buffer and incidence lists */
-    int genotypes_per_warp; /* ligands of at most 32 atoms (with matching rounds, at most 26
-                              torsions, one warp a genotype's atoms): 0 = two genotypes a
-                              warp, their arithmetic in packed FP32x2 instructions (the
-                              default), 1 = one genotype a warp */
+    int genotypes_per_warp; /* 0 (the default): two genotypes searched together, their
+                              arithmetic in packed FP32x2 instructions - a warp for ligands of
+                              at most 32 atoms (with matching rounds, at most 26 torsions, one
+                              warp a genotype's atoms), a block (ring sweep of the pairs) for
+                              larger ones where neither threads_per_pose nor poses_per_block
+                              nor pair_rounds asks for another form; 1: one genotype a warp or
+                              group of warps */
 } adgb_options;
 
 /* Receptor grid (Sec. 2.1: the receptor is fixed; its interaction with a
@@ -414,7 +417,8 @@ int rescore_fp64_dev(adgb_ctx *ctx, int receptor_id, int ligand_id, const float 
  *   over j < i.  The batch refers to the ligands and receptors: release the
  *   batch before them.  Errors: EINVAL, ENOTFOUND, ENOMEM.
  * batch_autotune - times the candidate launch shapes (32, 64 or 128 threads
- *   a genotype; poses per block; reduction variant) on this batch with
+ *   a genotype; poses per block; reduction variant; for ligands above 32
+ *   atoms two genotypes a 128-thread block) on this batch with
  *   `iters` evaluations per genotype from genes_dev (read on the context's
  *   own stream after the caller's work is complete; not modified), keeps the
  *   fastest for this batch and for later batches of the same size class

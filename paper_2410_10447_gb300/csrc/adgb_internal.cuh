@@ -14,6 +14,8 @@ constexpr float MS_EPS0 = 78.4f;
 constexpr float MS_B = MS_EPS0 - MS_A;
 constexpr float MS_LAMBDA = 0.003627f;
 constexpr float MS_K = 7.7839f;
+// scale of the pair term's reciprocal (pair_term.cuh) and so of the tables' Coulomb constants
+constexpr float PT_CSCALE = -1.0f / (MS_LAMBDA * MS_B * MS_B);
 
 constexpr int MAX_GENES = 6 + ADGB_MAX_TORS;
 constexpr int PAIR_CHUNK = 1024;   // pairs per force-buffer chunk (fixed: a ligand's arithmetic
@@ -62,6 +64,10 @@ struct LigDev {
                               // << 16 | hb << 24 | source used << 25, << 26
     const float4 *rconst;     // [n_rounds][r_lanes] the pair's constants as in pconst (zeros:
                               // no pair)
+    const float4 *ring;       // pair constants in the order of the ring sweep (ring_shape;
+                              // [warp][step][a][lane]; H-bond flag: the sign of A), or null
+                              // offset with ring_n = 0
+    int ring_n;               // its entries
     // the caller's per-type parameters, kept for the FP64 rescoring
     const float *t_R, *t_eps, *t_vol, *t_sol;
     const int *t_hb;
@@ -214,6 +220,70 @@ __host__ __device__ inline bool pair_eligible(int n_atoms, int n_tors, int n_pai
            (n_pairs == 0 || (n_rounds > 0 && r_lanes == 32));
 }
 
+// Ring sweep of the intramolecular pairs of ligands of 33 to 256 atoms: atoms
+// 0..N-1, padded with ghosts to np = a x la, form a ring; lane l of a team
+// holds atoms a l .. a l + a - 1 and at step s (1, 2, ..) meets atom a l + s,
+// which is at ring distance s - i from its i-th atom: steps 1 .. np/2 + a - 1
+// meet every pair once or more (the table lists it at one meeting).  Teams of
+// la <= 32 lanes: as many as fit a warp, every team of every warp taking a
+// slice of the steps.  Larger la: the warps cover the lanes in windows of 32,
+// and sets of `windows` warps take slices of the steps.
+struct RingShape {
+    int a, la, np;        // atoms a lane, lanes, ring length
+    int windows, teams;   // warps the lanes span; teams a warp
+    int warps;            // warps of the block
+    int slices, steps;    // slices of the steps, steps of a slice
+    int pos_len;          // positions the sweep reads (the ring and its continuation)
+    int copy_len, copies; // entries of a force copy (index: ring atom minus the slice's first
+                          // step), and copies: one a team, or one a warp with windows
+};
+// a = 3 or 5 (odd: no bank conflicts), whichever leaves fewer idle lanes at
+// N atoms; 4 warps (3 where the lanes span three windows).
+__host__ __device__ inline RingShape ring_shape(int N) {
+    RingShape r;
+    r.a = N <= 48 ? 3 : (N <= 80 ? 5 : (N <= 96 ? 3 : (N <= 160 ? 5 : 3)));
+    r.la = (N + r.a - 1) / r.a;
+    r.np = r.a * r.la;
+    r.windows = (r.la + 31) / 32;
+    r.teams = r.windows > 1 ? 1 : 32 / r.la;
+    r.warps = r.windows == 3 ? 3 : 4;
+    r.slices = r.windows > 1 ? r.warps / r.windows : r.teams * r.warps;
+    const int s = r.np / 2 + r.a - 1;
+    r.steps = (s + r.slices - 1) / r.slices;
+    r.pos_len = r.a * (r.la - 1) + r.slices * r.steps + 1;
+    r.copy_len = r.steps > r.a ? r.np - r.a + r.steps : r.np;
+    r.copies = r.windows > 1 ? r.warps : r.teams * r.warps;
+    return r;
+}
+// Slice of the steps whose reactions copy c holds.
+__host__ __device__ inline int ring_slice(const RingShape &r, int c) {
+    return r.windows > 1 ? c / r.windows : c;
+}
+// A lane's place: ring lane l, first step s0, force copy.
+struct RingLane {
+    int l, s0, copy;
+    bool active;   // an idle lane repeats lane 0 with zero constants and stores nothing
+};
+__host__ __device__ inline RingLane ring_lane(const RingShape &r, int warp, int lane) {
+    RingLane q;
+    int slice;
+    if (r.windows > 1) {
+        q.l = 32 * (warp % r.windows) + lane;
+        q.active = q.l < r.la;
+        q.copy = warp;
+        slice = warp / r.windows;
+    } else {
+        const int u = lane / r.la;
+        q.active = u < r.teams;
+        q.l = lane - u * r.la;
+        slice = q.copy = warp * r.teams + (q.active ? u : 0);
+    }
+    if (!q.active) q.l = 0;
+    q.s0 = 1 + slice * r.steps;
+    return q;
+}
+constexpr int RING_MIN_ATOMS = 33;
+
 // Threads a genotype by ligand size (one warp up to 32 atoms, two up to 56,
 // else 128; measured on 3000 genotypes, see the local-search launch-shape
 // sweep): the single-ligand calls and the serving loop's size classes alike.
@@ -249,6 +319,7 @@ struct EvalCfg {
     int chunk;      // pairs per force-buffer chunk
     int stage_pairs;  // copy the pair list and incidence lists to shared memory
     int paired;     // two genotypes a warp where the ligand is eligible (pair_eligible)
+    int ring;       // ring sweep, two genotypes a block, where the ligand has its table
 };
 
 // Carveout hint for the two-genotypes-a-warp kernels of the shuffle and
@@ -292,6 +363,18 @@ cudaError_t launch_eval_pair(const RecDev &rec, const LigDev &lig, const EvalCfg
                              const float *genes_in, float *genes_out, int n, int iters, float rho,
                              float eps, int resume, float *energy, float *grad, float *state,
                              cudaStream_t s, const int *iters_per_pose);
+// Ring sweep, two genotypes a block (ligands with a ring table; EvalCfg::ring).
+cudaError_t launch_eval_ring(const RecDev &rec, const LigDev &lig, const EvalCfg &cfg, int mode,
+                             const float *genes_in, float *genes_out, int n, int iters, float rho,
+                             float eps, int resume, float *energy, float *grad, float *state,
+                             cudaStream_t s, const int *iters_per_pose);
+// The same over work items of at most two genotypes, one a block; every
+// ligand has ring_shape's a and warps, layout_bytes the largest of theirs.
+cudaError_t launch_eval_ring_items(const WorkItem *items, int n_items, const LigDev *ligs,
+                                   const RecDev *recs, int a, int warps, int layout_bytes,
+                                   int variant, cudaStream_t s);
+int ring_layout_bytes(int n_atoms, int n_tors, int variant);
+cudaError_t ring_tc_gave_up_async(unsigned int *dst, cudaStream_t s);
 int pair_smem_bytes(int layout_bytes, int warps, int variant, int device);
 // Measurement-only paired local search without the steps in `skip`
 // (ls_ablation_dev); cudaErrorInvalidValue for masks or variants not built.
@@ -301,8 +384,9 @@ cudaError_t launch_pair_ablation(const RecDev &rec, const LigDev &lig, const Eva
 int pair_layout_bytes(int n_atoms, int n_tors, int ppb, int variant);
 // Queues copies of the tensor-core give-up counts of the local-search kernels
 // on the current device (dst[0]: one genotype a warp and Solis-Wets, dst[1]:
-// two genotypes a warp; monotonic) into host memory dst.
-cudaError_t tc_gave_up_async(unsigned int dst[2], cudaStream_t s);
+// two genotypes a warp, dst[2]: ring sweep; monotonic) into host memory dst.
+constexpr int TC_COUNTS = 3;
+cudaError_t tc_gave_up_async(unsigned int dst[TC_COUNTS], cudaStream_t s);
 cudaError_t pair_tc_gave_up_async(unsigned int *dst, cudaStream_t s);
 int pair_items_grid(const EvalCfg &cfg, int budget, int device);
 cudaError_t launch_eval_pair_items(const WorkItem *items, int n_items, const LigDev *ligs,

@@ -34,6 +34,12 @@ struct Ligand {
 namespace {
 // An uneven batch: items of (receptor, ligand, genotype count) run by one
 // persistent multi-ligand launch replayed from a captured CUDA graph.
+struct ItemClass {
+    EvalCfg cfg;            // launch shape of the class
+    int ring_a, ring_warps; // ring sweep (0: not)
+    int first, count;       // its items
+    int cost, budget, grid; // largest item, layout bytes, persistent blocks
+};
 struct Batch {
     std::vector<int> rec_idx, lig_idx, n_poses;  // per item, indices into the tables
     std::vector<LigDev> ligs;                    // unique ligands
@@ -44,17 +50,22 @@ struct Batch {
     RecDev *d_recs = nullptr;
     int *d_counter = nullptr;                    // [2], re-armed by the kernel
     WorkItem *d_items = nullptr;
-    int items_cap = 0, n_items = 0;
+    int items_cap = 0;
+    std::vector<ItemClass> classes;  // of the uploaded items
     EvalCfg cfg{32, 4, 0, 1, 0};
     bool tuned = false;
     cudaGraphExec_t exec = nullptr;
     // what the captured graph was built for
     const float *k_genes = nullptr;
     const float *k_energy = nullptr;
-    int k_iters = -1, k_tpp = 0, k_ppb = 0, k_var = -1, k_paired = -1, budget = 0, grid = 0;
+    int k_iters = -1, k_tpp = 0, k_ppb = 0, k_var = -1, k_paired = -1, k_ring = -1;
     float k_rho = 0.f, k_eps = 0.f;
 };
 }  // namespace
+
+// Kinds of launches a batch may need: one a class of ring shapes (a = 3 or 5
+// with 4 warps, a = 3 with 3), two genotypes a warp, one genotype a warp.
+constexpr int BATCH_CLASSES = 5;
 
 struct adgb_ctx {
     int device = 0;
@@ -66,6 +77,8 @@ struct adgb_ctx {
     int next_id = 1;
     std::string err;
     cudaStream_t stream = nullptr;  // used by the host-pointer calls
+    cudaStream_t side[BATCH_CLASSES - 1] = {};  // a batch's classes beside the first (made on first use)
+    cudaEvent_t fork = nullptr, join[BATCH_CLASSES - 1] = {};
     void *stage = nullptr;          // device staging for host-pointer calls
     size_t stage_bytes = 0;
     unsigned int tc_seen = 0;       // tensor-core give-up count already reported (device-wide)
@@ -104,10 +117,11 @@ int cuda_fail(adgb_ctx *c, cudaError_t e, const char *what) {
 // The device's tensor-core give-up count (both local-search modules), read
 // after everything queued on the context's stream.
 cudaError_t tc_count(adgb_ctx *c, unsigned int *count) {
-    unsigned int h[2] = {0, 0};
+    unsigned int h[TC_COUNTS] = {};
     cudaError_t e = tc_gave_up_async(h, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    *count = h[0] + h[1];
+    *count = 0;
+    for (unsigned int n : h) *count += n;
     return e;
 }
 
@@ -193,6 +207,7 @@ struct HostLigand {
     int R = 0, VP = 0;               // matching rounds, lanes a round
     std::vector<uint32_t> rword;     // [R][VP]
     std::vector<float4> rconst;      // [R][VP]
+    std::vector<float4> ring;        // pair constants in the order of the ring sweep
     std::vector<float> tR, teps, tvol, tsol;
     std::vector<int> thb;
     int max_type = 0;
@@ -391,6 +406,41 @@ void build_rounds(HostLigand &h) {
             wd[l] = w;
         }
     }
+}
+
+// Pair constants in the order of the ring sweep (RingShape): a pair listed
+// more than once has its constants added (the pair term is linear in them).
+void build_ring(HostLigand &h) {
+    const int N = h.N;
+    std::vector<float4> c((size_t)N * N, make_float4(0.f, 0.f, 0.f, 0.f));
+    std::vector<char> hb((size_t)N * N, 0);
+    for (int p = 0; p < h.NP; p++) {
+        const int i = h.pairs[p] & 255, j = (h.pairs[p] >> 8) & 255;
+        for (const size_t at : {(size_t)i * N + j, (size_t)j * N + i}) {
+            const float4 &k = h.pconst[p];
+            c[at] = make_float4(c[at].x + k.x, c[at].y + k.y, c[at].z + k.z, c[at].w + k.w);
+            hb[at] = (h.pairs[p] >> 24) & 1;
+        }
+    }
+    const RingShape r = ring_shape(N);
+    h.ring.assign((size_t)r.warps * r.steps * r.a * 32, make_float4(0.f, 0.f, 0.f, 0.f));
+    for (int w = 0; w < r.warps; w++)
+        for (int lane = 0; lane < 32; lane++) {
+            const RingLane q = ring_lane(r, w, lane);
+            if (!q.active) continue;
+            for (int t = 0; t < r.steps; t++)
+                for (int a = 0; a < r.a; a++) {
+                    const int i = r.a * q.l + a, d = q.s0 + t - a, j = (i + d) % r.np;
+                    // each pair at one of its meetings: ring distance 1 .. np/2,
+                    // an opposite pair (distance np/2, np even) from its first atom
+                    if (d < 1 || d > r.np / 2 || i >= N || j >= N) continue;
+                    if (r.np % 2 == 0 && d == r.np / 2 && i >= r.np / 2) continue;
+                    float4 k = c[(size_t)i * N + j];
+                    if (hb[(size_t)i * N + j]) k.x = -k.x;
+                    k.z *= PT_CSCALE;
+                    h.ring[(((size_t)w * r.steps + t) * r.a + a) * 32 + lane] = k;
+                }
+        }
 }
 
 // Whether the kernels use the matching rounds of a ligand (mode as
@@ -736,6 +786,9 @@ EvalCfg adgb::launch_cfg(const LigDev &L, int tpp_opt, int ppb_opt, int variant,
     cfg.ppb = ppb;
     cfg.paired = genotypes_per_warp == 0 &&
                  pair_eligible(L.n_atoms, L.n_tors, L.n_pairs, L.n_rounds, L.r_lanes, cfg.tpp);
+    // above 32 atoms the ring sweep, two genotypes a block, unless the caller
+    // set a launch shape or asked for one genotype a warp
+    cfg.ring = genotypes_per_warp == 0 && tpp_opt == 0 && ppb_opt == 0 && L.ring_n > 0;
     return cfg;
 }
 
@@ -789,6 +842,10 @@ int make_ligand_blob(std::string *err, const adgb_ligand_desc *d, int pair_round
     const size_t o_incoff = take(4 * (size_t)(NCH > 0 ? NCH : 1) * (N + 1)), o_inc = take(2 * 2 * (size_t)NPz);
     const size_t RVz = h.R > 0 ? (size_t)h.R * h.VP : 1;
     const size_t o_rword = take(4 * RVz), o_rconst = take(16 * RVz);
+    // the ring sweep: every ligand above 32 atoms, unless the caller asked for
+    // the force buffer
+    if (N >= RING_MIN_ATOMS && pair_rounds == 0) build_ring(h);
+    const size_t o_ring = take(16 * std::max<size_t>(h.ring.size(), 1));
     const size_t o_tR = take(4 * NT), o_teps = take(4 * NT), o_tvol = take(4 * NT),
                  o_tsol = take(4 * NT), o_thb = take(4 * NT);
     std::vector<unsigned char> &buf = out.bytes;
@@ -813,6 +870,7 @@ int make_ligand_blob(std::string *err, const adgb_ligand_desc *d, int pair_round
         memcpy(&buf[o_rword], h.rword.data(), 4 * (size_t)h.R * h.VP);
         memcpy(&buf[o_rconst], h.rconst.data(), 16 * (size_t)h.R * h.VP);
     }
+    if (!h.ring.empty()) memcpy(&buf[o_ring], h.ring.data(), 16 * h.ring.size());
     memcpy(&buf[o_tR], h.tR.data(), 4 * NT);
     memcpy(&buf[o_teps], h.teps.data(), 4 * NT);
     memcpy(&buf[o_tvol], h.tvol.data(), 4 * NT);
@@ -844,6 +902,8 @@ int make_ligand_blob(std::string *err, const adgb_ligand_desc *d, int pair_round
     v.inc = reinterpret_cast<const uint16_t *>(at(o_inc));
     v.rword = reinterpret_cast<const uint32_t *>(at(o_rword));
     v.rconst = reinterpret_cast<const float4 *>(at(o_rconst));
+    v.ring = reinterpret_cast<const float4 *>(at(o_ring));
+    v.ring_n = (int)h.ring.size();
     v.t_R = reinterpret_cast<const float *>(at(o_tR));
     v.t_eps = reinterpret_cast<const float *>(at(o_teps));
     v.t_vol = reinterpret_cast<const float *>(at(o_tvol));
@@ -874,6 +934,7 @@ LigDev bind_ligand(const LigandBlob &b, const unsigned char *mem) {
     v.inc = mv(v.inc);
     v.rword = mv(v.rword);
     v.rconst = mv(v.rconst);
+    v.ring = mv(v.ring);
     v.t_R = mv(v.t_R);
     v.t_eps = mv(v.t_eps);
     v.t_vol = mv(v.t_vol);
@@ -1001,6 +1062,11 @@ int adgb_destroy(adgb_ctx *c) {
         for (auto &kv : c->recs) cudaFree(kv.second.cells);
         for (auto &kv : c->ligs) cudaFree(kv.second.mem);
         if (c->stage) cudaFree(c->stage);
+        for (cudaStream_t t : c->side)
+            if (t) cudaStreamDestroy(t);
+        for (cudaEvent_t e : c->join)
+            if (e) cudaEventDestroy(e);
+        if (c->fork) cudaEventDestroy(c->fork);
         if (c->stream) cudaStreamDestroy(c->stream);
     }
     delete c;
@@ -1665,34 +1731,72 @@ extern "C" int dock_noalloc_dev(adgb_ctx *c, int receptor_id, int ligand_id,
 // ---------------------------------------------------------------------------
 namespace {
 
-int batch_budget(const Batch &b, const EvalCfg &cfg) {
-    int budget = 1024;
-    for (size_t u = 0; u < b.ligs.size(); u++)
-        budget = std::max(budget, items_layout_bytes(cfg, b.lig_n[u], b.lig_t[u], b.lig_np[u]));
-    return budget;
-}
-
 // Two genotypes a warp only when every ligand of the batch qualifies (one
-// launch shape serves the whole batch).
+// launch shape serves the whole batch, unless the ring sweep is on).
 bool batch_pairable(const Batch &b, const EvalCfg &cfg) {
     for (const LigDev &l : b.ligs)
         if (!pair_eligible(l.n_atoms, l.n_tors, l.n_pairs, l.n_rounds, l.r_lanes, cfg.tpp)) return false;
     return true;
 }
 
-// Items of ppb genotypes of one ligand, longest (most work) first.
+// Whether any ligand of the batch has a ring table (the ring sweep then runs
+// those, and the smaller ones run two genotypes a warp where they qualify).
+bool batch_ringable(const Batch &b) {
+    for (const LigDev &l : b.ligs)
+        if (l.ring_n > 0) return true;
+    return false;
+}
+
+// Launch shape of a ligand in a batch of shape cfg, and its ring class.
+EvalCfg item_cfg(const LigDev &l, const EvalCfg &cfg, int *ring_a, int *ring_warps) {
+    *ring_a = *ring_warps = 0;
+    EvalCfg e = cfg;
+    e.ring = 0;
+    if (!cfg.ring) return e;
+    e.tpp = 32;
+    e.ppb = 4;
+    e.paired = pair_eligible(l.n_atoms, l.n_tors, l.n_pairs, l.n_rounds, l.r_lanes, 32);
+    if (l.ring_n > 0) {
+        const RingShape r = ring_shape(l.n_atoms);
+        e.ring = 1;
+        e.paired = 0;
+        e.ppb = 2;
+        *ring_a = r.a;
+        *ring_warps = r.warps;
+    }
+    return e;
+}
+
+// Items of ppb genotypes of one ligand by class of launch, the class with the
+// longest items first, and longest (most work) first within it.
 std::vector<WorkItem> batch_items(const Batch &b, const EvalCfg &cfg, float *genes, float *energy,
-                                  int iters, float rho, float eps) {
-    std::vector<WorkItem> items;
+                                  int iters, float rho, float eps, std::vector<ItemClass> &classes) {
+    classes.clear();
+    std::vector<int> cls(b.ligs.size());
+    for (size_t u = 0; u < b.ligs.size(); u++) {
+        ItemClass k{};
+        k.cfg = item_cfg(b.ligs[u], cfg, &k.ring_a, &k.ring_warps);
+        size_t q = 0;
+        while (q < classes.size() &&
+               !(classes[q].ring_a == k.ring_a && classes[q].ring_warps == k.ring_warps &&
+                 classes[q].cfg.paired == k.cfg.paired))
+            q++;
+        if (q == classes.size()) classes.push_back(k);
+        cls[u] = (int)q;
+        const int bytes = k.ring_a ? ring_layout_bytes(b.lig_n[u], b.lig_t[u], cfg.variant)
+                                   : items_layout_bytes(k.cfg, b.lig_n[u], b.lig_t[u], b.lig_np[u]);
+        classes[q].budget = std::max(std::max(classes[q].budget, 1024), bytes);
+    }
+    std::vector<std::pair<int, WorkItem>> items;
     long long row = 0;
     for (size_t i = 0; i < b.n_poses.size(); i++) {
-        const int u = b.lig_idx[i];
+        const int u = b.lig_idx[i], ppb = classes[cls[u]].cfg.ppb;
         const int cost = (int)std::min<long long>(INT32_MAX, (long long)(b.lig_np[u] + 8 * b.lig_n[u] + 64));
-        for (int k = 0; k < b.n_poses[i]; k += cfg.ppb) {
+        for (int k = 0; k < b.n_poses[i]; k += ppb) {
             WorkItem w;
             w.lig = u;
             w.rec = b.rec_idx[i];
-            w.count = std::min(cfg.ppb, b.n_poses[i] - k);
+            w.count = std::min(ppb, b.n_poses[i] - k);
             w.gstride = 6 + ADGB_MAX_TORS;
             w.genes = genes + (row + k) * (long long)(6 + ADGB_MAX_TORS);
             w.energy = energy + row + k;
@@ -1701,14 +1805,35 @@ std::vector<WorkItem> batch_items(const Batch &b, const EvalCfg &cfg, float *gen
             w.cost = cost;
             w.rho = rho;
             w.eps = eps;
-            items.push_back(w);
+            items.push_back({cls[u], w});
+            classes[cls[u]].cost = std::max(classes[cls[u]].cost, cost);
+            classes[cls[u]].count++;
         }
         row += b.n_poses[i];
     }
-    std::stable_sort(items.begin(), items.end(), [](const WorkItem &x, const WorkItem &y) {
-        return x.cost > y.cost || (x.cost == y.cost && x.lig < y.lig);
+    // classes without items (ligands with no genotypes) launch nothing
+    std::vector<int> order;
+    for (size_t q = 0; q < classes.size(); q++)
+        if (classes[q].count > 0) order.push_back((int)q);
+    std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return classes[x].cost > classes[y].cost; });
+    std::vector<int> rank(classes.size(), 0);
+    std::vector<ItemClass> kept;
+    int first = 0;
+    for (int q : order) {
+        rank[q] = (int)kept.size();
+        kept.push_back(classes[q]);
+        kept.back().first = first;
+        first += classes[q].count;
+    }
+    classes = kept;
+    std::stable_sort(items.begin(), items.end(), [&](const auto &x, const auto &y) {
+        if (rank[x.first] != rank[y.first]) return rank[x.first] < rank[y.first];
+        return x.second.cost > y.second.cost || (x.second.cost == y.second.cost && x.second.lig < y.second.lig);
     });
-    return items;
+    std::vector<WorkItem> out;
+    out.reserve(items.size());
+    for (const auto &it : items) out.push_back(it.second);
+    return out;
 }
 
 cudaError_t upload_items(Batch &b, const std::vector<WorkItem> &items, cudaStream_t s) {
@@ -1719,10 +1844,53 @@ cudaError_t upload_items(Batch &b, const std::vector<WorkItem> &items, cudaStrea
         if (e != cudaSuccess) return e;
         b.items_cap = (int)items.size();
     }
-    b.n_items = (int)items.size();
     cudaError_t e = cudaMemcpyAsync(b.d_items, items.data(), sizeof(WorkItem) * items.size(),
                                     cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e;
+}
+
+// Persistent grids of the classes that use one; false if a shape fits no SM.
+bool batch_grids(Batch &b, int device) {
+    for (ItemClass &k : b.classes) {
+        if (k.ring_a) continue;
+        k.grid = items_grid(k.cfg, k.budget, device);
+        if (k.grid < 1) return false;
+    }
+    return true;
+}
+
+// Launches every class of the batch's uploaded items, the first on `s`, the
+// others on the context's side streams between a fork and a join on `s`, so
+// that a class's last blocks overlap with the next class's first.
+cudaError_t launch_batch(adgb_ctx *c, Batch &b, cudaStream_t s) {
+    const int n = (int)b.classes.size();
+    cudaError_t e = cudaSuccess;
+    if (n > 1) {
+        if (!c->fork) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
+        for (int q = 0; q < n - 1 && e == cudaSuccess; q++) {
+            if (!c->side[q]) e = cudaStreamCreateWithFlags(&c->side[q], cudaStreamNonBlocking);
+            if (e == cudaSuccess && !c->join[q])
+                e = cudaEventCreateWithFlags(&c->join[q], cudaEventDisableTiming);
+        }
+        if (e == cudaSuccess) e = cudaEventRecord(c->fork, s);
+    }
+    for (int q = 0; q < n && e == cudaSuccess; q++) {
+        const ItemClass &k = b.classes[q];
+        const cudaStream_t t = q == 0 ? s : c->side[q - 1];
+        if (q > 0) e = cudaStreamWaitEvent(t, c->fork, 0);
+        if (e != cudaSuccess) break;
+        const WorkItem *items = b.d_items + k.first;
+        e = k.ring_a ? launch_eval_ring_items(items, k.count, b.d_ligs, b.d_recs, k.ring_a,
+                                              k.ring_warps, k.budget, k.cfg.variant, t)
+                     : launch_eval_items(items, k.count, b.d_ligs, b.d_recs, b.d_counter + 2 * q,
+                                         k.cfg, k.budget, k.grid, t);
+        if (q > 0) {   // join also after a failed launch, so that a capture can end
+            cudaError_t j = cudaEventRecord(c->join[q - 1], t);
+            if (j == cudaSuccess) j = cudaStreamWaitEvent(s, c->join[q - 1], 0);
+            if (e == cudaSuccess) e = j;
+        }
+    }
     return e;
 }
 
@@ -1769,10 +1937,10 @@ extern "C" int batch_create(adgb_ctx *c, int n_items, const int *receptor_ids, c
     DeviceGuard g(c->device);
     cudaError_t e = cudaMalloc(&b.d_ligs, sizeof(LigDev) * b.ligs.size());
     if (e == cudaSuccess) e = cudaMalloc(&b.d_recs, sizeof(RecDev) * b.recs.size());
-    if (e == cudaSuccess) e = cudaMalloc(&b.d_counter, 2 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMalloc(&b.d_counter, 2 * BATCH_CLASSES * sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(b.d_ligs, b.ligs.data(), sizeof(LigDev) * b.ligs.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b.d_recs, b.recs.data(), sizeof(RecDev) * b.recs.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(b.d_counter, 0, 2 * sizeof(int));
+    if (e == cudaSuccess) e = cudaMemset(b.d_counter, 0, 2 * BATCH_CLASSES * sizeof(int));
     if (e != cudaSuccess) {
         cudaFree(b.d_ligs);
         cudaFree(b.d_recs);
@@ -1781,6 +1949,8 @@ extern "C" int batch_create(adgb_ctx *c, int n_items, const int *receptor_ids, c
     }
     b.cfg.variant = c->opts.reduce_variant;
     b.cfg.paired = c->opts.genotypes_per_warp == 0;
+    // the ring sweep unless the context set a launch shape
+    b.cfg.ring = b.cfg.paired && c->opts.threads_per_pose == 0 && c->opts.poses_per_block == 0;
     if (c->opts.threads_per_pose > 0) {   // the context's launch shape, until tuned
         b.cfg.tpp = c->opts.threads_per_pose;
         b.cfg.ppb = c->opts.poses_per_block > 0 ? c->opts.poses_per_block : 128 / b.cfg.tpp;
@@ -1827,24 +1997,23 @@ extern "C" int batch_local_search_dev(adgb_ctx *c, int batch_id, float *genes_de
     EvalCfg cfg = b.cfg;
     if (!b.tuned || p->reduce_variant >= 0) cfg.variant = variant;
     cfg.paired = cfg.paired && batch_pairable(b, cfg);
+    cfg.ring = cfg.ring && batch_ringable(b);
     cudaError_t e = cudaSuccess;
     const bool same = b.exec && b.k_genes == genes_dev && b.k_energy == best_energy_dev &&
                       b.k_iters == p->iters && b.k_rho == p->rho && b.k_eps == p->eps &&
                       b.k_tpp == cfg.tpp && b.k_ppb == cfg.ppb && b.k_var == cfg.variant &&
-                      b.k_paired == cfg.paired;
+                      b.k_paired == cfg.paired && b.k_ring == cfg.ring;
     if (!same) {
         if (b.exec) cudaGraphExecDestroy(b.exec);
         b.exec = nullptr;
-        b.budget = batch_budget(b, cfg);
-        b.grid = items_grid(cfg, b.budget, c->device);
-        if (b.grid < 1) return fail(c, ADGB_EINVAL, "batch_local_search: launch shape does not fit an SM");
-        e = upload_items(b, batch_items(b, cfg, genes_dev, best_energy_dev, p->iters, p->rho, p->eps),
-                         c->stream);
+        const std::vector<WorkItem> items =
+            batch_items(b, cfg, genes_dev, best_energy_dev, p->iters, p->rho, p->eps, b.classes);
+        if (!batch_grids(b, c->device)) return fail(c, ADGB_EINVAL, "batch_local_search: launch shape does not fit an SM");
+        e = upload_items(b, items, c->stream);
         cudaGraph_t graph = nullptr;
         if (e == cudaSuccess) e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            cudaError_t el = launch_eval_items(b.d_items, b.n_items, b.d_ligs, b.d_recs, b.d_counter,
-                                               cfg, b.budget, b.grid, c->stream);
+            const cudaError_t el = launch_batch(c, b, c->stream);
             e = cudaStreamEndCapture(c->stream, &graph);
             if (el != cudaSuccess) e = el;
         }
@@ -1860,6 +2029,7 @@ extern "C" int batch_local_search_dev(adgb_ctx *c, int batch_id, float *genes_de
         b.k_ppb = cfg.ppb;
         b.k_var = cfg.variant;
         b.k_paired = cfg.paired;
+        b.k_ring = cfg.ring;
     }
     e = cudaGraphLaunch(b.exec, (cudaStream_t)stream);
     return e == cudaSuccess ? ADGB_OK : cuda_fail(c, e, "batch_local_search: graph launch");
@@ -1873,17 +2043,21 @@ extern "C" int batch_autotune(adgb_ctx *c, int batch_id, const float *genes_dev,
     Batch &b = it->second;
     if (iters < 1 || (b.total > 0 && !genes_dev)) return fail(c, ADGB_EINVAL, "batch_autotune: bad arguments");
     DeviceGuard g(c->device);
-    // one genotype a warp (the last field 0) and, where every ligand of the
-    // batch qualifies, two genotypes a warp
+    // one genotype a warp (the last field 0); where every ligand of the batch
+    // qualifies, two genotypes a warp; where any has a ring table, the ring
+    // sweep for those and two genotypes a warp for the smaller ones
     const EvalCfg all[] = {{32, 4, ADGB_REDUCE_SHFL, 1, 0, 0}, {32, 4, ADGB_REDUCE_MMA_TF32X2, 1, 0, 0},
                            {32, 4, ADGB_REDUCE_MMA_BF16X3, 1, 0, 0}, {32, 4, ADGB_REDUCE_TCGEN05, 1, 0, 0},
                            {32, 2, ADGB_REDUCE_SHFL, 1, 0, 0}, {64, 2, ADGB_REDUCE_SHFL, 1, 0, 0},
                            {128, 1, ADGB_REDUCE_SHFL, 1, 0, 0},
                            {32, 4, ADGB_REDUCE_SHFL, 1, 0, 1}, {32, 8, ADGB_REDUCE_SHFL, 1, 0, 1},
-                           {32, 4, ADGB_REDUCE_TCGEN05, 1, 0, 1}, {32, 8, ADGB_REDUCE_TCGEN05, 1, 0, 1}};
+                           {32, 4, ADGB_REDUCE_TCGEN05, 1, 0, 1}, {32, 8, ADGB_REDUCE_TCGEN05, 1, 0, 1},
+                           {128, 2, ADGB_REDUCE_SHFL, 1, 0, 0, 1}, {128, 2, ADGB_REDUCE_TCGEN05, 1, 0, 0, 1}};
     std::vector<EvalCfg> cands;
     for (const EvalCfg &cf : all)
-        if (!cf.paired || (c->opts.genotypes_per_warp == 0 && batch_pairable(b, cf))) cands.push_back(cf);
+        if (c->opts.genotypes_per_warp == 0 ? (!cf.paired || batch_pairable(b, cf)) && (!cf.ring || batch_ringable(b))
+                                            : !cf.paired && !cf.ring)
+            cands.push_back(cf);
     const size_t gbytes = sizeof(float) * (size_t)b.total * (6 + ADGB_MAX_TORS);
     float *tg = nullptr, *te = nullptr;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1895,17 +2069,14 @@ extern "C" int batch_autotune(adgb_ctx *c, int batch_id, const float *genes_dev,
     EvalCfg best{};
     for (const EvalCfg &cfg : cands) {
         if (e != cudaSuccess) break;
-        const int budget = batch_budget(b, cfg);
-        const int grid = items_grid(cfg, budget, c->device);
-        if (grid < 1) continue;
+        const std::vector<WorkItem> items = batch_items(b, cfg, tg, te, iters, 0.8f, 1e-2f, b.classes);
+        if (!batch_grids(b, c->device)) continue;
         float ms_min = INFINITY;
         for (int rep = 0; rep < 2 && e == cudaSuccess; rep++) {
             e = cudaMemcpyAsync(tg, genes_dev, gbytes, cudaMemcpyDeviceToDevice, c->stream);
-            if (e == cudaSuccess) e = upload_items(b, batch_items(b, cfg, tg, te, iters, 0.8f, 1e-2f), c->stream);
+            if (e == cudaSuccess && rep == 0) e = upload_items(b, items, c->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-            if (e == cudaSuccess)
-                e = launch_eval_items(b.d_items, b.n_items, b.d_ligs, b.d_recs, b.d_counter, cfg, budget,
-                                      grid, c->stream);
+            if (e == cudaSuccess) e = launch_batch(c, b, c->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float ms = 0.f;
@@ -1935,7 +2106,7 @@ extern "C" int batch_autotune(adgb_ctx *c, int batch_id, const float *genes_dev,
         chosen->poses_per_block = best.ppb;
         chosen->reduce_variant = best.variant;
         chosen->pair_rounds = c->opts.pair_rounds;
-        chosen->genotypes_per_warp = best.paired ? 0 : 1;
+        chosen->genotypes_per_warp = best.paired || best.ring ? 0 : 1;
     }
     return ADGB_OK;
 }

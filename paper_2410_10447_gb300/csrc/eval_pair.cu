@@ -33,6 +33,7 @@
 #include <math.h>
 
 #include "adgb_internal.cuh"
+#include "packed.cuh"
 #include "reduce.cuh"
 #include "tcgen05.cuh"
 
@@ -71,31 +72,8 @@ enum {
 };
 constexpr int TC2_TEST_LIMIT = 64;   // mbarrier probes of SK_NOISSUE's waits
 
-// ------------------------------------------------------- packed FP32x2
-__device__ __forceinline__ float2 bc(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, bc(-1.f), a); }
-
-struct V2 {   // a 3-vector of both genotypes
-    float2 x, y, z;
-};
-
 __device__ __forceinline__ float2 shfl2(float2 v, int src) {
     return make_float2(__shfl_sync(FULL, v.x, src), __shfl_sync(FULL, v.y, src));
-}
-
-// a x b of both genotypes
-__device__ __forceinline__ V2 cross2(const V2 &a, const V2 &b) {
-    V2 c;
-    c.x = fma2(a.y, b.z, mul2(bc(-1.f), mul2(a.z, b.y)));
-    c.y = fma2(a.z, b.x, mul2(bc(-1.f), mul2(a.x, b.z)));
-    c.z = fma2(a.x, b.y, mul2(bc(-1.f), mul2(a.y, b.x)));
-    return c;
-}
-__device__ __forceinline__ float2 dot2(const V2 &a, const V2 &b) {
-    return fma2(a.z, b.z, fma2(a.y, b.y, mul2(a.x, b.x)));
 }
 
 // p += s (k x v) + omc (k x (k x v)), v = p - b, for both genotypes: the
@@ -437,19 +415,6 @@ struct PairArgs {
     float *state;
     const int *iters_pp;
     int n, iters, resume, mode, ppb;
-    float rho, eps;
-};
-
-// Inputs and outputs of the warp's two genotypes (pointers at each one).
-struct PairIO {
-    const float *genes_in[2];
-    float *genes_out[2];
-    float *energy[2];
-    float *grad[2];
-    float *state[2];
-    int iters[2];
-    int nvalid;   // 1: the second genotype is a copy of the first, not written
-    int mode, resume;
     float rho, eps;
 };
 

@@ -1,0 +1,727 @@
+// Fused scoring / ADADELTA local search of ligands of more than 32 atoms
+// (Sec. 2.1, Sec. 3; Table 1's gpu_gradient_minAD): one block of 3 or 4
+// warps searches two genotypes, packed (genotype A in .x, B in .y), so that
+// the ligand's pair constants, torsion tree and addresses are read and
+// computed once for both.
+//
+// The intramolecular pairs are swept as a ring (RingShape): a lane holds A
+// consecutive atoms of both genotypes in registers, and at step s meets atom
+// j = A lane + s of the ring, computing its A pairs with it.  In a step every
+// lane's j is another atom, so the reaction on j is added to the warp's own
+// copy of the forces in shared memory without atomics: two loads, two stores
+// and a warp barrier for A pairs of two genotypes.  A odd puts a quarter
+// warp's 16-byte accesses into different banks without padding.  The steps
+// are split over the block's warps (and, for small ligands, over two or three
+// teams of lanes in a warp); every atom's owner then sums the copies.  The
+// pair constants come from a table in the order of the sweep (coalesced
+// 16-byte loads), zeros for pairs that are not listed, the H-bond flag in the
+// sign of A.
+//
+// What bounds it: from ~90 atoms on, the issue and FMA pipe of the pair terms
+// (26 packed and 14 scalar instructions for a pair of two genotypes, 15 more
+// for distances, sums and the reaction; 256 atoms: FMA pipe 50%, issue 46%,
+// LSU data pipe 31% busy, the rest fixed latencies at 10-15 warps an SM); below
+// that, the latency of an evaluation's seven barriers, torsion walk and grid
+// loads.  The kernel it took over from for these ligands (one genotype a 64-
+// or 128-thread group, forces through per-pair slots in shared memory) had its
+// LSU data pipe 73% busy at 256 atoms, 46% of the shared-memory wavefronts
+// bank-conflict replays, at 107K warp instructions an evaluation; this one
+// issues 45K.  Local search, M evaluations/s before -> with the sweep:
+// 45 atoms x 1000 genotypes 95 -> 156, 90 x 1500 31 -> 84, 128 x 8000
+// 17 -> 41, 192 x 6000 10 -> 27, 256 x 2048 6.2 -> 12.0, x 8192 6.8 -> 14.
+//
+// Per evaluation (block barriers between the steps):
+//   1. gene threads publish genes and sin / (1 - cos) of every angle;
+//   2. a thread an atom and genotype: torsion walk, grid terms, and the sums
+//      of (E, g, torque) of the grid terms: pair forces are central and
+//      cancel in the rigid-body sums exactly, so they take no part in them;
+//   3. ring sweep; 4. atoms' total gradients;
+//   5. torsions' moving-set sums (8 lanes a torsion) and the reduction;
+//   6. gene gradient, best tracking and ADADELTA by the gene threads.
+#include <math.h>
+
+#include <algorithm>
+
+#include "adgb_internal.cuh"
+#include "eval_common.cuh"
+#include "packed.cuh"
+#include "pair_term.cuh"
+#include "reduce.cuh"
+
+namespace adgb {
+
+namespace {
+
+constexpr unsigned FULL = 0xffffffffu;
+
+// Shared-memory layout of one block: the ligand's constants, then the two
+// genotypes' working arrays.  Offsets in bytes, 16-byte aligned.
+struct RingSmem {
+    int ref, type, frag, tparent, tatoms, taxis, tbref;
+    int pxy, pz;        // positions [pos_len]: (xA, xB, yA, yB) and (zA, zB)
+    int cxy, cz;        // force copies [copies][copy_len], as the positions
+    int gxy, gz;        // atoms' gradients [N], as the positions
+    int genes, sc, ggrad, red, stage;
+    int ada;            // gene threads' state [MAX_GENES][4]: E[g^2], E[d^2], best, Omega
+    int total;
+    RingShape r;
+
+    __host__ __device__ inline void make(int N, int T, bool mma_stage) {
+        r = ring_shape(N);
+        auto al16 = [](int x) { return (x + 15) & ~15; };
+        const int Tn = T > 0 ? T : 1;
+        int o = 0;
+        ref = o;     o = al16(o + 16 * N);
+        type = o;    o = al16(o + 4 * N);
+        frag = o;    o = al16(o + 4 * N);
+        tparent = o; o = al16(o + 4 * Tn);
+        tatoms = o;  o = al16(o + 16 * Tn);
+        taxis = o;   o = al16(o + 16 * Tn);
+        tbref = o;   o = al16(o + 16 * Tn);
+        pxy = o;     o = al16(o + 16 * r.pos_len);
+        pz = o;      o = al16(o + 8 * r.pos_len);
+        cxy = o;     o = al16(o + 16 * r.copies * r.copy_len);
+        cz = o;      o = al16(o + 8 * r.copies * r.copy_len);
+        gxy = o;     o = al16(o + 16 * N);
+        gz = o;      o = al16(o + 8 * N);
+        genes = o;   o = al16(o + 8 * MAX_GENES);
+        sc = o;      o = al16(o + 16 * (ADGB_MAX_TORS + 4));
+        ggrad = o;   o = al16(o + 8 * MAX_GENES);
+        red = o;     o = al16(o + 4 * 16 * r.warps);
+        ada = o;     o = al16(o + 32 * MAX_GENES);
+        stage = o;   o = al16(o + (mma_stage ? 4 * 32 * 12 * r.warps : 0));
+        total = o;
+    }
+};
+
+struct RingArgs {
+    RecDev rec;
+    LigDev lig;
+    RingSmem L;
+    const float *genes_in;
+    float *genes_out;
+    float *energy;
+    float *grad;
+    float *state;
+    const int *iters_pp;
+    int n, iters, resume, mode;
+    float rho, eps;
+};
+
+__device__ __forceinline__ void stage_ring_ligand(unsigned char *sm, const RingSmem &L,
+                                                  const LigDev &lig) {
+    const int N = lig.n_atoms, T = lig.n_tors;
+    float4 *s_ref = reinterpret_cast<float4 *>(sm + L.ref);
+    int *s_type = reinterpret_cast<int *>(sm + L.type);
+    int *s_frag = reinterpret_cast<int *>(sm + L.frag);
+    int *s_tpar = reinterpret_cast<int *>(sm + L.tparent);
+    int4 *s_tat = reinterpret_cast<int4 *>(sm + L.tatoms);
+    float4 *s_tax = reinterpret_cast<float4 *>(sm + L.taxis);
+    float4 *s_tb = reinterpret_cast<float4 *>(sm + L.tbref);
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        s_ref[i] = lig.ref[i];
+        s_type[i] = lig.type[i];
+        s_frag[i] = lig.frag[i];
+    }
+    for (int k = threadIdx.x; k < T; k += blockDim.x) {
+        s_tpar[k] = lig.tparent[k];
+        s_tat[k] = lig.tatoms[k];
+        s_tax[k] = lig.taxis[k];
+        s_tb[k] = lig.tbref[k];
+    }
+}
+
+__device__ __forceinline__ V2 load_v2(const float4 *xy, const float2 *z, int i) {
+    const float4 a = xy[i];
+    return {make_float2(a.x, a.y), make_float2(a.z, a.w), z[i]};
+}
+
+// Sums a warp's 8 values of the lane's own genotype (its parity) over the
+// lanes of the same parity: reduce-scatter over lane bits 4..2, a butterfly
+// over bit 1; lane (c2 c1 c0 0 g) ends with component c of genotype g.
+__device__ __forceinline__ float reduce_parity8(float v[8]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int lv = 0; lv < 3; lv++) {
+        const int h = 4 >> lv, m = 16 >> lv;
+        const bool up = lane & m;
+#pragma unroll
+        for (int k = 0; k < h; k++) {
+            const float send = up ? v[k] : v[k + h];
+            const float keep = up ? v[k + h] : v[k];
+            v[k] = keep + __shfl_xor_sync(FULL, send, m);
+        }
+    }
+    return v[0] + __shfl_xor_sync(FULL, v[0], 2);
+}
+
+// Whole evaluation loop of a block's two genotypes (all threads).
+template <int A, int VAR>
+__device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L, const LigDev &lig,
+                                            const RecDev &rec, const PairIO &io, Tc05Warp &tw) {
+    const int t = threadIdx.x, TH = blockDim.x, lane = t & 31, warp = t >> 5;
+    const int N = lig.n_atoms, T = lig.n_tors, G = 6 + T;
+    const RingShape &rs = L.r;
+    const float4 *s_ref = reinterpret_cast<const float4 *>(sm + L.ref);
+    const int *s_type = reinterpret_cast<const int *>(sm + L.type);
+    const int *s_frag = reinterpret_cast<const int *>(sm + L.frag);
+    const int *s_tpar = reinterpret_cast<const int *>(sm + L.tparent);
+    const int4 *s_tat = reinterpret_cast<const int4 *>(sm + L.tatoms);
+    const float4 *s_tax = reinterpret_cast<const float4 *>(sm + L.taxis);
+    const float4 *s_tb = reinterpret_cast<const float4 *>(sm + L.tbref);
+    float4 *pxy = reinterpret_cast<float4 *>(sm + L.pxy);
+    float2 *pz = reinterpret_cast<float2 *>(sm + L.pz);
+    float4 *cxy = reinterpret_cast<float4 *>(sm + L.cxy);
+    float2 *cz = reinterpret_cast<float2 *>(sm + L.cz);
+    float4 *gxy = reinterpret_cast<float4 *>(sm + L.gxy);
+    float2 *gz = reinterpret_cast<float2 *>(sm + L.gz);
+    float2 *genes_s = reinterpret_cast<float2 *>(sm + L.genes);
+    float4 *sc = reinterpret_cast<float4 *>(sm + L.sc);
+    float2 *ggrad = reinterpret_cast<float2 *>(sm + L.ggrad);
+    float *red = reinterpret_cast<float *>(sm + L.red);   // [warp][genotype][8]
+    float *stage = reinterpret_cast<float *>(sm + L.stage) + warp * 32 * 12;
+
+    // the thread's gene (j = t) of both genotypes, and ADADELTA state
+    const int j = t;
+    float2 om = bc(0.f), eg2 = bc(0.f), ed2 = bc(0.f);
+    if (j < G) {
+#pragma unroll
+        for (int g = 0; g < 2; g++) {
+            float o, a = 0.f, b = 0.f;
+            if (io.resume) {
+                const float *st = io.state[g];
+                o = st[j];
+                a = st[G + j];
+                b = st[2 * G + j];
+            } else {
+                o = io.genes_in[g][j];
+            }
+            if (g == 0) {
+                om.x = o; eg2.x = a; ed2.x = b;
+            } else {
+                om.y = o; eg2.y = a; ed2.y = b;
+            }
+        }
+    }
+    // (between evaluations it lives in shared memory: the ring sweep needs the
+    // registers)
+    float2 *ada = reinterpret_cast<float2 *>(sm + L.ada) + 4 * min(j, MAX_GENES - 1);
+    if (j < G) {
+        ada[0] = eg2;
+        ada[1] = ed2;
+        ada[2] = ada[3] = om;
+    }
+    __syncthreads();
+    float2 best_e = bc(INFINITY);
+    // the lane's place in the ring sweep
+    const RingLane rl = ring_lane(rs, warp, lane);
+    const int copy0 = rl.copy * rs.copy_len + A * rl.l;   // slot of step 0 in the lane's copy
+    const int pos0 = A * rl.l + rl.s0;
+    const float4 *table = lig.ring + (size_t)warp * rs.steps * A * 32 + lane;
+    // the thread's genotype in steps 2 and 5 (blockDim.x is even)
+    const int gen = t & 1;
+    const int iters = max(io.iters[0], io.iters[1]);
+
+    for (int it = 0; it < iters; it++) {
+        // 1. genes and sin / (1 - cos) of every angle, a thread a gene and
+        //    genotype (half-angle form: exact zero at a zero angle; phi and
+        //    theta as (sin, cos) of the angle)
+        if (t < 2 * G) {
+            const int jj = t >> 1;
+            const float om = reinterpret_cast<const float *>(sm + L.ada)[8 * jj + 6 + gen];
+            const bool full = jj == 3 || jj == 4;
+            float sn, cs;
+            sincosf(full ? om : 0.5f * om, &sn, &cs);
+            reinterpret_cast<float *>(genes_s)[2 * jj + gen] = om;
+            const float2 w = full ? make_float2(sn, cs) : make_float2(2.f * sn * cs, 2.f * sn * sn);
+            float2 *sc2 = reinterpret_cast<float2 *>(sc) + gen;
+            if (jj >= 6) sc2[2 * (jj - 6)] = w;
+            else if (jj >= 3) sc2[2 * (SC_ROT + jj - 3)] = w;
+        }
+        __syncthreads();
+
+        // 2. coordinates and grid terms of the thread's atoms in its genotype
+        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        {
+            const float *gs = reinterpret_cast<const float *>(genes_s) + gen;
+            const float2 *sc2 = reinterpret_cast<const float2 *>(sc) + gen;   // [2 k + genotype]
+            const float3 tr = make_float3(gs[0], gs[2], gs[4]);
+            const float2 sphi = sc2[2 * SC_ROT], sth = sc2[2 * SC_ROT + 2], sal = sc2[2 * SC_ROT + 4];
+            const float3 u = make_float3(sth.x * sphi.y, sth.x * sphi.x, sth.y);
+            // R - I = sin(a) [u]x + (1 - cos(a)) (u u^T - I)
+            const float s = sal.x, o = sal.y;
+            const float m00 = o * (u.x * u.x - 1.f), m11 = o * (u.y * u.y - 1.f),
+                        m22 = o * (u.z * u.z - 1.f);
+            const float m01 = o * u.x * u.y - s * u.z, m10 = o * u.x * u.y + s * u.z;
+            const float m02 = o * u.x * u.z + s * u.y, m20 = o * u.x * u.z - s * u.y;
+            const float m12 = o * u.y * u.z - s * u.x, m21 = o * u.y * u.z + s * u.x;
+            for (int i = t >> 1; i < N; i += TH >> 1) {
+                const float4 r4 = s_ref[i];
+                float3 p = make_float3(r4.x, r4.y, r4.z);
+                for (int k = s_frag[i]; k >= 0;) {
+                    const int up = s_tpar[k];   // read ahead of the rotation's chain
+                    rotate_about(p, s_tax[k], s_tb[k], sc2[2 * k]);
+                    k = up;
+                }
+                float3 x, g;
+                x.x = p.x + (m00 * p.x + m01 * p.y + m02 * p.z) + tr.x;
+                x.y = p.y + (m10 * p.x + m11 * p.y + m12 * p.z) + tr.y;
+                x.z = p.z + (m20 * p.x + m21 * p.y + m22 * p.z) + tr.z;
+                float *xyf = reinterpret_cast<float *>(pxy), *zf = reinterpret_cast<float *>(pz);
+                auto put = [&](int q) {
+                    xyf[4 * q + gen] = x.x;
+                    xyf[4 * q + 2 + gen] = x.y;
+                    zf[2 * q + gen] = x.z;
+                };
+                for (int q = i; q < rs.pos_len; q += rs.np) put(q);
+                if (i == 0)   // the ring's ghosts past the last atom (no listed pairs)
+                    for (int a = N; a < rs.np; a++)
+                        for (int q = a; q < rs.pos_len; q += rs.np) put(q);
+                v[0] += inter_atom(rec, s_type[i], r4.w, x, g);
+                float *gxf = reinterpret_cast<float *>(gxy), *gzf = reinterpret_cast<float *>(gz);
+                gxf[4 * i + gen] = g.x;
+                gxf[4 * i + 2 + gen] = g.y;
+                gzf[2 * i + gen] = g.z;
+                const float3 d = make_float3(x.x - tr.x, x.y - tr.y, x.z - tr.z);
+                v[1] += g.x;
+                v[2] += g.y;
+                v[3] += g.z;
+                v[4] += d.y * g.z - d.z * g.y;
+                v[5] += d.z * g.x - d.x * g.z;
+                v[6] += d.x * g.y - d.y * g.x;
+            }
+        }
+        // sums of the grid terms (shuffle form: over the warp right away)
+        if constexpr (VAR == ADGB_REDUCE_SHFL) {
+            const float mine = reduce_parity8(v);
+            if ((lane & 2) == 0) red[16 * warp + 8 * gen + (lane >> 2)] = mine;
+        }
+        // the warp's copies of the forces start from zero
+        for (int q = lane; q < rs.teams * rs.copy_len; q += 32) {
+            const int c = warp * rs.teams * rs.copy_len + q;
+            cxy[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+            cz[c] = bc(0.f);
+        }
+        __syncthreads();
+
+        // 3. ring sweep
+        float2 e_pair = bc(0.f);
+        if (lig.n_pairs > 0) {
+            V2 xi[A], fi[A];
+#pragma unroll
+            for (int a = 0; a < A; a++) {
+                xi[a] = load_v2(pxy, pz, A * rl.l + a);
+                fi[a] = {bc(0.f), bc(0.f), bc(0.f)};
+            }
+            const float4 *tp = table;
+#pragma unroll 2
+            for (int st = 0; st < rs.steps; st++, tp += A * 32) {
+                const V2 xj = load_v2(pxy, pz, pos0 + st);
+                V2 fj = {bc(0.f), bc(0.f), bc(0.f)};
+#pragma unroll
+                for (int a = 0; a < A; a++) {
+                    const float4 pc = __ldg(tp + 32 * a);
+                    const bool hb = __float_as_int(pc.x) < 0;
+                    const V2 d = {sub2(xi[a].x, xj.x), sub2(xi[a].y, xj.y), sub2(xi[a].z, xj.z)};
+                    const float2 r2 = fma2(d.z, d.z, fma2(d.y, d.y, mul2(d.x, d.x)));
+                    float2 ft;
+                    const float2 e = pair_terms2(r2, bc(fabsf(pc.x)), bc(pc.y), bc(pc.z), bc(pc.w),
+                                                 {hb, hb}, ft);
+                    e_pair = add2(e_pair, e);
+                    fi[a] = {fma2(ft, d.x, fi[a].x), fma2(ft, d.y, fi[a].y), fma2(ft, d.z, fi[a].z)};
+                    fj = {fma2(ft, d.x, fj.x), fma2(ft, d.y, fj.y), fma2(ft, d.z, fj.z)};
+                }
+                const V2 c = load_v2(cxy, cz, copy0 + st);
+                if (rl.active) {
+                    const V2 n = {sub2(c.x, fj.x), sub2(c.y, fj.y), sub2(c.z, fj.z)};
+                    cxy[copy0 + st] = make_float4(n.x.x, n.x.y, n.y.x, n.y.y);
+                    cz[copy0 + st] = n.z;
+                }
+                __syncwarp();   // the next step's slots were other lanes' in this one
+            }
+            // the lane's own atoms: slot of atom i is i - s0 around the ring
+#pragma unroll
+            for (int a = 0; a < A; a++) {
+                int q = A * rl.l + a - rl.s0;
+                if (q < 0) q += rs.np;
+                q += rl.copy * rs.copy_len;
+                if (rl.active) {
+                    const V2 c = load_v2(cxy, cz, q);
+                    const V2 n = {add2(c.x, fi[a].x), add2(c.y, fi[a].y), add2(c.z, fi[a].z)};
+                    cxy[q] = make_float4(n.x.x, n.x.y, n.y.x, n.y.y);
+                    cz[q] = n.z;
+                }
+            }
+        }
+        __syncthreads();
+
+        // 4. atoms' total gradients: grid terms and every copy's pair forces
+        if (lig.n_pairs > 0 && T > 0) {
+            for (int i = t; i < N; i += TH) {
+                V2 g = load_v2(gxy, gz, i);
+#pragma unroll 4
+                for (int c = 0; c < rs.copies; c++) {
+                    int q = i - 1 - ring_slice(rs, c) * rs.steps;
+                    if (q < 0) q += rs.np;
+                    const V2 f = load_v2(cxy, cz, c * rs.copy_len + q);
+                    g = {add2(g.x, f.x), add2(g.y, f.y), add2(g.z, f.z)};
+                    if (q + rs.np < rs.copy_len) {   // at most one more turn (copy_len < 2 np)
+                        const V2 h = load_v2(cxy, cz, c * rs.copy_len + q + rs.np);
+                        g = {add2(g.x, h.x), add2(g.y, h.y), add2(g.z, h.z)};
+                    }
+                }
+                gxy[i] = make_float4(g.x.x, g.x.y, g.y.x, g.y.y);
+                gz[i] = g.z;
+            }
+            __syncthreads();
+        }
+
+        // 5. torsion gradients, 8 lanes a torsion: a . sum (x - x_b) x g over
+        //    the moving atoms (one contiguous range), both genotypes
+        for (int k0 = 0; k0 < T; k0 += TH >> 3) {
+            const int k = k0 + (t >> 3);
+            V2 acc = {bc(0.f), bc(0.f), bc(0.f)};
+            int4 ta = make_int4(0, 0, 0, 0);
+            V2 xb = acc;
+            if (k < T) {
+                ta = s_tat[k];
+                xb = load_v2(pxy, pz, ta.y);
+                for (int i = ta.z + (t & 7); i < ta.w; i += 8) {
+                    const V2 g = load_v2(gxy, gz, i), x = load_v2(pxy, pz, i);
+                    const V2 d = {sub2(x.x, xb.x), sub2(x.y, xb.y), sub2(x.z, xb.z)};
+                    const V2 c = cross2(d, g);
+                    acc = {add2(acc.x, c.x), add2(acc.y, c.y), add2(acc.z, c.z)};
+                }
+            }
+#pragma unroll
+            for (int off = 4; off > 0; off >>= 1) {
+                acc.x.x += __shfl_xor_sync(FULL, acc.x.x, off);
+                acc.x.y += __shfl_xor_sync(FULL, acc.x.y, off);
+                acc.y.x += __shfl_xor_sync(FULL, acc.y.x, off);
+                acc.y.y += __shfl_xor_sync(FULL, acc.y.y, off);
+                acc.z.x += __shfl_xor_sync(FULL, acc.z.x, off);
+                acc.z.y += __shfl_xor_sync(FULL, acc.z.y, off);
+            }
+            if (k < T && (t & 7) == 0) {
+                float2 gk = bc(0.f);
+                if (ta.w > ta.z) {
+                    const V2 xa = load_v2(pxy, pz, ta.x);
+                    const V2 ax = {sub2(xb.x, xa.x), sub2(xb.y, xa.y), sub2(xb.z, xa.z)};
+                    const float2 l2 = dot2(ax, ax);
+                    gk = mul2(dot2(ax, acc), make_float2(rsqrtf(l2.x), rsqrtf(l2.y)));
+                }
+                ggrad[6 + k] = gk;
+            }
+        }
+        // the pair energies of the lane's own genotype: its own and its
+        // partner lane's; in the shuffle form summed over the warp and added to
+        // the grid energy, else reduced with the grid sums on the tensor cores
+        float ep = gen ? e_pair.y : e_pair.x;
+        ep += __shfl_xor_sync(FULL, gen ? e_pair.x : e_pair.y, 1);
+        if constexpr (VAR == ADGB_REDUCE_SHFL) {
+#pragma unroll
+            for (int off = 16; off > 1; off >>= 1) ep += __shfl_xor_sync(FULL, ep, off);
+            if (lane < 2) red[16 * warp + 8 * gen] += ep;
+        } else {
+            v[0] += ep;
+#pragma unroll
+            for (int g = 0; g < 2; g++) {
+                float w[8];
+#pragma unroll
+                for (int c = 0; c < 8; c++) w[c] = gen == g ? v[c] : 0.f;
+                if constexpr (VAR == ADGB_REDUCE_TCGEN05) warp_sum8_tc05(w, tw);
+                else warp_sum8<VAR>(w, stage);
+                if (lane == 0) {
+#pragma unroll
+                    for (int c = 0; c < 8; c++) red[16 * warp + 8 * g + c] = w[c];
+                }
+            }
+        }
+        // what the gene formulas take from this evaluation's genes, read
+        // before the barrier after which they may be rewritten
+        const float4 c_phi = sc[SC_ROT], c_th = sc[SC_ROT + 1], c_al = sc[SC_ROT + 2];
+        __syncthreads();
+
+        // 6. gene gradient, best tracking, ADADELTA
+        if (j < G) {
+            auto total = [&](int c) {
+                float2 s = make_float2(red[c], red[8 + c]);
+                for (int w = 1; w < rs.warps; w++)
+                    s = add2(s, make_float2(red[16 * w + c], red[16 * w + 8 + c]));
+                return s;
+            };
+            const float2 E = total(0);
+            float2 gj;
+            if (j < 3) {
+                gj = total(1 + j);
+            } else if (j < 6) {
+                // d u / d phi or d theta; angular velocity sin(a) du + (1-cos a) u x du
+                const float2 sphi = make_float2(c_phi.x, c_phi.z), cphi = make_float2(c_phi.y, c_phi.w);
+                const float2 sth = make_float2(c_th.x, c_th.z), cth = make_float2(c_th.y, c_th.w);
+                const float2 s = make_float2(c_al.x, c_al.z), o = make_float2(c_al.y, c_al.w);
+                const V2 u = {mul2(sth, cphi), mul2(sth, sphi), cth};
+                const bool th = j == 4;
+                const V2 du = {th ? mul2(cth, cphi) : mul2(bc(-1.f), mul2(sth, sphi)),
+                               th ? mul2(cth, sphi) : mul2(sth, cphi),
+                               th ? mul2(bc(-1.f), sth) : bc(0.f)};
+                const V2 uxd = cross2(u, du);
+                const V2 wv = {fma2(s, du.x, mul2(o, uxd.x)), fma2(s, du.y, mul2(o, uxd.y)),
+                               fma2(s, du.z, mul2(o, uxd.z))};
+                const V2 tq = {total(4), total(5), total(6)};
+                gj = dot2(tq, j == 5 ? u : wv);
+            } else {
+                gj = ggrad[j];
+            }
+            if (io.mode == MODE_SCORE) {
+                if (j == 0) {
+                    io.energy[0][0] = E.x;
+                    if (io.nvalid > 1) io.energy[1][0] = E.y;
+                }
+                if (io.grad[0]) io.grad[0][j] = gj.x;
+                if (io.nvalid > 1 && io.grad[1]) io.grad[1][j] = gj.y;
+            } else {
+                float2 eg2 = ada[0], ed2 = ada[1], om = ada[3];
+                const bool act_a = it < io.iters[0], act_b = it < io.iters[1];
+                if (act_a && E.x < best_e.x) {
+                    best_e.x = E.x;
+                    ada[2].x = om.x;
+                }
+                if (act_b && E.y < best_e.y) {
+                    best_e.y = E.y;
+                    ada[2].y = om.y;
+                }
+                const float2 rho = bc(io.rho), omr = bc(1.f - io.rho), ep = bc(io.eps);
+                const float2 neg2 = fma2(rho, eg2, mul2(omr, mul2(gj, gj)));
+                const float2 a2 = add2(ed2, ep), b2 = add2(neg2, ep);
+                const float2 d = mul2(mul2(make_float2(-sqrtf(a2.x), -sqrtf(a2.y)),
+                                           make_float2(rsqrtf(b2.x), rsqrtf(b2.y))), gj);
+                const float2 ned2 = fma2(rho, ed2, mul2(omr, mul2(d, d)));
+                float2 w = add2(om, d);
+                if (j >= 6) {
+                    w.x -= 2.f * PI_F * floorf((w.x + PI_F) * (0.5f / PI_F));
+                    w.y -= 2.f * PI_F * floorf((w.y + PI_F) * (0.5f / PI_F));
+                }
+                if (act_a) {
+                    eg2.x = neg2.x;
+                    ed2.x = ned2.x;
+                    om.x = w.x;
+                }
+                if (act_b) {
+                    eg2.y = neg2.y;
+                    ed2.y = ned2.y;
+                    om.y = w.y;
+                }
+                ada[0] = eg2;
+                ada[1] = ed2;
+                ada[3] = om;
+            }
+        }
+        if (io.mode == MODE_SCORE) return;
+        __syncthreads();   // the updated genes are published by other threads
+    }
+    if (io.mode == MODE_SCORE || j >= G) return;
+    const float2 best = ada[2];
+    eg2 = ada[0];
+    ed2 = ada[1];
+    om = ada[3];
+#pragma unroll
+    for (int g = 0; g < 2; g++) {
+        if (g >= io.nvalid) break;
+        io.genes_out[g][j] = g ? best.y : best.x;
+        if (io.state[g]) {
+            float *st = io.state[g];
+            st[j] = g ? om.y : om.x;
+            st[G + j] = g ? eg2.y : eg2.x;
+            st[2 * G + j] = g ? ed2.y : ed2.x;
+        }
+        if (j == 0) io.energy[g][0] = g ? best_e.y : best_e.x;
+    }
+}
+
+// Resident blocks of 128 threads an SM the kernels are built for (MB): 4, at
+// 128 registers a thread, or 5 at 96, which spill a little outside the sweep.
+// 5 for a = 3 up to 96 atoms where the launch fills more than 4 blocks an SM
+// (12 000 genotypes of 45 atoms 176 -> 186M evaluations/s, of 90 atoms 84.0 ->
+// 86.4M; 1500 of 90 atoms, one wave instead of two, 67 -> 80M); where 4 blocks
+// an SM hold the launch they run 3% faster (45 atoms x 1000), and above 160
+// atoms shared memory allows no fifth (256 atoms 13.7 -> 12.2M).
+template <int A, int VAR, int MB>
+__global__ void __launch_bounds__(128, MB) eval_ring_kernel(const RingArgs a) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    unsigned char *sm = smem_raw + tc_front<VAR>();
+    stage_ring_ligand(sm, a.L, a.lig);
+    Tc05Warp tw;
+    tc_begin<VAR>(smem_raw, tw);
+    __syncthreads();
+    const int G = 6 + a.lig.n_tors, p0 = 2 * blockIdx.x;
+    PairIO io;
+    io.nvalid = min(2, a.n - p0);
+#pragma unroll
+    for (int g = 0; g < 2; g++) {
+        const size_t p = p0 + (g < io.nvalid ? g : 0);
+        io.genes_in[g] = a.genes_in ? a.genes_in + p * G : nullptr;
+        io.genes_out[g] = a.genes_out ? a.genes_out + p * G : nullptr;
+        io.energy[g] = a.energy + p;
+        io.grad[g] = a.grad ? a.grad + p * G : nullptr;
+        io.state[g] = a.state ? a.state + p * 3 * G : nullptr;
+        io.iters[g] = a.mode == MODE_SCORE ? 1 : (a.iters_pp ? a.iters_pp[p] : a.iters);
+    }
+    io.mode = a.mode;
+    io.resume = a.resume;
+    io.rho = a.rho;
+    io.eps = a.eps;
+    search_ring<A, VAR>(sm, a.L, a.lig, a.rec, io, tw);
+    tc_end<VAR>(tw);
+}
+
+// Multi-ligand form (batches): block b searches work item b (up to two
+// genotypes of one ligand); the host orders the items longest first and every
+// ligand of the launch has this a and number of warps.
+template <int A, int VAR>
+__global__ void __launch_bounds__(128, 4) eval_ring_items_kernel(const WorkItem *items,
+                                                                 const LigDev *ligs,
+                                                                 const RecDev *recs) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    __shared__ RingSmem L;
+    unsigned char *sm = smem_raw + tc_front<VAR>();
+    const WorkItem w = items[blockIdx.x];
+    const LigDev &lig = ligs[w.lig];
+    if (threadIdx.x == 0) L.make(lig.n_atoms, lig.n_tors, uses_mma_stage(VAR));
+    __syncthreads();
+    stage_ring_ligand(sm, L, lig);
+    Tc05Warp tw;
+    tc_begin<VAR>(smem_raw, tw);
+    __syncthreads();
+    PairIO io;
+    io.nvalid = w.count;
+#pragma unroll
+    for (int g = 0; g < 2; g++) {
+        const int k = g < io.nvalid ? g : 0;
+        io.genes_in[g] = w.genes + (size_t)k * w.gstride;
+        io.genes_out[g] = w.genes + (size_t)k * w.gstride;
+        io.energy[g] = w.energy + k;
+        io.grad[g] = nullptr;
+        io.state[g] = nullptr;
+        io.iters[g] = w.iters ? w.iters[k] : w.iters_all;
+    }
+    io.mode = MODE_LS;
+    io.resume = 0;
+    io.rho = w.rho;
+    io.eps = w.eps;
+    search_ring<A, VAR>(sm, L, lig, recs[w.rec], io, tw);
+    tc_end<VAR>(tw);
+}
+
+template <int A, int VAR, int MB>
+cudaError_t launch_ring_t(const RingArgs &a, int threads, int smem, cudaStream_t s) {
+    auto k = eval_ring_kernel<A, VAR, MB>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k<<<(a.n + 1) / 2, threads, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <int A, int MB>
+cudaError_t launch_ring_v(const RingArgs &a, int variant, int threads, int smem, cudaStream_t s) {
+    switch (variant) {
+        case ADGB_REDUCE_SHFL: return launch_ring_t<A, ADGB_REDUCE_SHFL, MB>(a, threads, smem, s);
+        case ADGB_REDUCE_MMA_TF32X2:
+            return launch_ring_t<A, ADGB_REDUCE_MMA_TF32X2, MB>(a, threads, smem, s);
+        case ADGB_REDUCE_MMA_BF16X3:
+            return launch_ring_t<A, ADGB_REDUCE_MMA_BF16X3, MB>(a, threads, smem, s);
+        case ADGB_REDUCE_TCGEN05:
+            return launch_ring_t<A, ADGB_REDUCE_TCGEN05, MB>(a, threads, smem, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+template <int A, int VAR>
+cudaError_t launch_ring_items_t(const WorkItem *items, int n_items, const LigDev *ligs,
+                                const RecDev *recs, int threads, int smem, cudaStream_t s) {
+    auto k = eval_ring_items_kernel<A, VAR>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k<<<n_items, threads, smem, s>>>(items, ligs, recs);
+    return cudaGetLastError();
+}
+
+template <int A>
+cudaError_t launch_ring_items_v(const WorkItem *items, int n_items, const LigDev *ligs,
+                                const RecDev *recs, int variant, int threads, int smem,
+                                cudaStream_t s) {
+    switch (variant) {
+        case ADGB_REDUCE_SHFL:
+            return launch_ring_items_t<A, ADGB_REDUCE_SHFL>(items, n_items, ligs, recs, threads, smem, s);
+        case ADGB_REDUCE_MMA_TF32X2:
+            return launch_ring_items_t<A, ADGB_REDUCE_MMA_TF32X2>(items, n_items, ligs, recs, threads, smem, s);
+        case ADGB_REDUCE_MMA_BF16X3:
+            return launch_ring_items_t<A, ADGB_REDUCE_MMA_BF16X3>(items, n_items, ligs, recs, threads, smem, s);
+        case ADGB_REDUCE_TCGEN05:
+            return launch_ring_items_t<A, ADGB_REDUCE_TCGEN05>(items, n_items, ligs, recs, threads, smem, s);
+    }
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+int ring_layout_bytes(int n_atoms, int n_tors, int variant) {
+    RingSmem L;
+    L.make(n_atoms, n_tors, uses_mma_stage(variant));
+    return L.total;
+}
+
+cudaError_t launch_eval_ring_items(const WorkItem *items, int n_items, const LigDev *ligs,
+                                   const RecDev *recs, int a, int warps, int layout_bytes,
+                                   int variant, cudaStream_t s) {
+    if (n_items == 0) return cudaSuccess;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const int smem = tc_smem_bytes(layout_bytes, warps, variant, dev);
+    if (smem < 0) return cudaErrorInvalidValue;
+    if (a == 3) return launch_ring_items_v<3>(items, n_items, ligs, recs, variant, 32 * warps, smem, s);
+    return launch_ring_items_v<5>(items, n_items, ligs, recs, variant, 32 * warps, smem, s);
+}
+
+cudaError_t launch_eval_ring(const RecDev &rec, const LigDev &lig, const EvalCfg &cfg, int mode,
+                             const float *genes_in, float *genes_out, int n, int iters, float rho,
+                             float eps, int resume, float *energy, float *grad, float *state,
+                             cudaStream_t s, const int *iters_per_pose) {
+    if (n == 0) return cudaSuccess;
+    RingArgs a;
+    a.rec = rec;
+    a.lig = lig;
+    a.L.make(lig.n_atoms, lig.n_tors, uses_mma_stage(cfg.variant));
+    const RingShape &rs = a.L.r;
+    a.genes_in = genes_in;
+    a.genes_out = genes_out;
+    a.energy = energy;
+    a.grad = grad;
+    a.state = state;
+    a.iters_pp = iters_per_pose;
+    a.n = n;
+    a.iters = iters;
+    a.resume = resume;
+    a.mode = mode;
+    a.rho = rho;
+    a.eps = eps;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const int smem = tc_smem_bytes(a.L.total, rs.warps, cfg.variant, dev);
+    if (smem < 0) return cudaErrorInvalidValue;
+    if (rs.a == 5) return launch_ring_v<5, 4>(a, cfg.variant, 32 * rs.warps, smem, s);
+    int sms = 0;
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if (lig.n_atoms <= 96 && (n + 1) / 2 > 4 * sms)
+        return launch_ring_v<3, 5>(a, cfg.variant, 32 * rs.warps, smem, s);
+    return launch_ring_v<3, 4>(a, cfg.variant, 32 * rs.warps, smem, s);
+}
+
+cudaError_t ring_tc_gave_up_async(unsigned int *dst, cudaStream_t s) {
+    return cudaMemcpyFromSymbolAsync(dst, g_tc_gave_up, sizeof(unsigned int), 0,
+                                     cudaMemcpyDeviceToHost, s);
+}
+
+}  // namespace adgb

@@ -211,8 +211,8 @@ void release_job(adgb_server *s, Job *j) {
     }
 }
 
-// The job's tensor-core give-up snapshots (pinned): [0..1] when its first
-// launch starts, [2..3] after its last.  The counts are device-wide, so a
+// The job's tensor-core give-up snapshots (pinned): [0 .. TC_COUNTS) when
+// its first launch starts, [TC_COUNTS .. 2 TC_COUNTS) after its last.  The counts are device-wide, so a
 // give-up in another job's kernels while this job ran fails this one too.
 unsigned int *tc_counts(const Job *j) {
     return (unsigned int *)((char *)j->res.p + al256(4 * (size_t)j->d.n_runs * j->G) +
@@ -231,7 +231,8 @@ cudaError_t setup_job(adgb_server *s, Job *j) {
     job_layout(*j, j->mem);
     const int runs = j->d.n_runs;
     j->cnt = pinned_take(s, IN_FLIGHT * (size_t)runs * 12 + j->blob.bytes.size());
-    j->res = pinned_take(s, al256(4 * (size_t)runs * j->G) + 16 * (size_t)runs + 16);
+    j->res = pinned_take(s, al256(4 * (size_t)runs * j->G) + 16 * (size_t)runs +
+                               2 * TC_COUNTS * sizeof(unsigned int));
     if (!j->cnt.p || !j->res.p) return cudaErrorMemoryAllocation;
     // the ligand blob through pinned memory (an asynchronous copy)
     unsigned char *stage = (unsigned char *)j->cnt.p + IN_FLIGHT * (size_t)runs * 12;
@@ -347,7 +348,7 @@ bool service(adgb_server *s, Job *j, bool *complete) {
             e = cudaMemcpyAsync(h_g, j->d_best_genes, 4 * (size_t)runs * j->G, cudaMemcpyDeviceToHost, j->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h_e, j->d_best_e, 8 * (size_t)runs, cudaMemcpyDeviceToHost, j->stream);
         if (e == cudaSuccess) e = cudaMemcpyAsync(h_v, j->w.evals, 8 * (size_t)runs, cudaMemcpyDeviceToHost, j->stream);
-        if (e == cudaSuccess) e = tc_gave_up_async(tc_counts(j) + 2, j->stream);
+        if (e == cudaSuccess) e = tc_gave_up_async(tc_counts(j) + TC_COUNTS, j->stream);
         if (e == cudaSuccess) e = cudaEventRecord(j->ev_fin, j->stream);
         if (e != cudaSuccess) {
             job_error(s, j, e);
@@ -361,7 +362,8 @@ bool service(adgb_server *s, Job *j, bool *complete) {
     if (q == cudaErrorNotReady) return progress;
     if (q != cudaSuccess) {
         job_error(s, j, q);
-    } else if (const unsigned int *tc = tc_counts(j); tc[0] + tc[1] != tc[2] + tc[3]) {
+    } else if (const unsigned int *tc = tc_counts(j);
+               !std::equal(tc, tc + TC_COUNTS, tc + TC_COUNTS)) {
         j->tc_failed = true;
         s->err = "serving: a tensor-core completion wait gave up while the job ran";
     } else {
@@ -567,7 +569,9 @@ int dock_submit(adgb_server *s, int receptor_id, const adgb_ligand_desc *lig,
     j->bytes = job_layout(*j, nullptr);
     {
         const double genotypes = (double)j->d.n_runs * j->d.pop;
-        const double warps = j->cfg.paired ? genotypes / 2 : genotypes * (j->cfg.tpp / 32);
+        const double warps = j->cfg.paired ? genotypes / 2
+                             : j->cfg.ring ? genotypes / 2 * ring_shape(j->blob.rel.n_atoms).warps
+                                           : genotypes * (j->cfg.tpp / 32);
         j->fill = warps / s->warps_gpu;
     }
     const size_t limit = s->budget > 0 ? s->budget
