@@ -47,7 +47,7 @@ struct LigDev {
     const float4 *tbref;      // [T] reference position of b
     const uint32_t *pairs;    // [Np] i | j << 8 | (ti*16+tj) << 16 | hb << 24
     const float2 *tptab;      // [256] (A, B): E = A r^-12 - B r^-m, m = 10 if hb else 6
-    const float4 *pconst;     // [Np] per pair, in pair order: (A, B, w_el 332.06 q_i q_j,
+    const float4 *pconst;     // [Np] per pair, in pair order: (A, B, PT_CSCALE w_el 332.06 q_i q_j,
                               // w_ds (S_i V_j + S_j V_i))
     const int *perm;          // [N] internal index -> caller's index
     int n_chunks;             // ceil(Np / PAIR_CHUNK)

@@ -437,7 +437,6 @@ void build_ring(HostLigand &h) {
                     if (r.np % 2 == 0 && d == r.np / 2 && i >= r.np / 2) continue;
                     float4 k = c[(size_t)i * N + j];
                     if (hb[(size_t)i * N + j]) k.x = -k.x;
-                    k.z *= PT_CSCALE;
                     h.ring[(((size_t)w * r.steps + t) * r.a + a) * 32 + lane] = k;
                 }
         }
@@ -744,7 +743,7 @@ int build_ligand(std::string *err, const adgb_ligand_desc *d, HostLigand &h) {
         const uint32_t c = h.pairs[p];
         const int i = c & 255, j = (c >> 8) & 255;
         const float2 ab = h.tptab[(c >> 16) & 255];
-        const double qq = (double)ADGB_W_EL * (double)ADGB_ELEC_KCAL * (double)h.ref[i].w * (double)h.ref[j].w;
+        const double qq = (double)PT_CSCALE * (double)ADGB_W_EL * (double)ADGB_ELEC_KCAL * (double)h.ref[i].w * (double)h.ref[j].w;
         const double ds = (double)h.sv[i].x * h.sv[j].y + (double)h.sv[j].x * h.sv[i].y;
         h.pconst[p] = make_float4(ab.x, ab.y, (float)qq, (float)ds);
     }

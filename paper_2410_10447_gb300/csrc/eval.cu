@@ -25,6 +25,7 @@
 
 #include "adgb_internal.cuh"
 #include "eval_common.cuh"
+#include "pair_term.cuh"
 #include "philox.cuh"
 #include "reduce.cuh"
 
@@ -44,9 +45,6 @@ struct EvalArgs {
     float rho, eps;
 };
 
-constexpr float INV_SIG2 = 1.0f / (ADGB_DS_SIGMA * ADGB_DS_SIGMA);
-constexpr float HALF_INV_SIG2 = 0.5f / (ADGB_DS_SIGMA * ADGB_DS_SIGMA);
-constexpr float RMIN2 = ADGB_R_MIN * ADGB_R_MIN;
 
 template <int TPP>
 __device__ __forceinline__ void group_sync(int group) {
@@ -57,92 +55,35 @@ __device__ __forceinline__ void group_sync(int group) {
     }
 }
 
-// One intramolecular pair: 12-6 (12-10 for donor-acceptor pairs) with
-// A r^-12 - B r^-m, Coulomb with the Mehler-Solmajer dielectric, and
-// desolvation.  pc = (A, B, w_el 332.06 q_i q_j, w_ds (S_i V_j + S_j V_i)).
-// Returns the energy; f = dE/dx_i (atom j gets -f).
-__device__ __forceinline__ float pair_term(float4 xi, float4 xj, float4 pc, bool hb, float3 &f) {
-    const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
-    const float r2 = dx * dx + dy * dy + dz * dz;
-    const bool live = r2 >= RMIN2;
-    const float r2c = fmaxf(r2, RMIN2);
-    const float rinv = rsqrtf(r2c);
-    const float rc = r2c * rinv;
-    const float r2i = rinv * rinv;
-    const float r6i = r2i * r2i * r2i;
-    const float r12i = r6i * r6i;
-    const float rmi = hb ? r6i * r2i * r2i : r6i;
-    const float m = hb ? 10.f : 6.f;
-    const float evdw = pc.x * r12i - pc.y * rmi;
-    const float dvdw = (-12.f * pc.x * r12i + m * pc.y * rmi) * rinv;
-    // eps(r) = num / den with den = 1 + k e^{-lambda B r}, num = A den + B;
-    // 1/eps = den^2 r and eps'/eps = B k lambda B e^{..} r with r = 1/(den num):
-    // one reciprocal for the whole dielectric.
-    const float C = pc.z;
-    const float ex = __expf(-MS_LAMBDA * MS_B * rc);
-    const float den = 1.f + MS_K * ex;
-    const float num = MS_A * den + MS_B;
-    const float rr = __fdividef(1.f, den * num);
-    const float eel = C * rinv * (den * den * rr);
-    const float del = -eel * (rinv + (MS_B * MS_K * MS_LAMBDA * MS_B) * ex * rr);
-    const float eds = pc.w * __expf(-r2 * HALF_INV_SIG2);
-    const float fr = live ? (dvdw + del) * rinv : 0.f;
-    const float fd = -eds * INV_SIG2;
-    f = make_float3((fr + fd) * dx, (fr + fd) * dy, (fr + fd) * dz);
-    return evdw + eel + eds;
-}
-
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float3 xyz3(float4 a) { return make_float3(a.x, a.y, a.z); }
-__device__ __forceinline__ float2 f2s(float a) { return make_float2(a, a); }
 
-// Two pair terms (a, b), the same formulas as pair_term with the adds,
-// multiplies and fused multiply-adds of both pairs in packed FP32x2
-// instructions (one instruction, two IEEE round-to-nearest results);
-// reciprocal square roots, exponentials, the reciprocal, compares and
-// selects per pair.  Returns the two energies' sum; fa, fb = dE/dx_i of each
-// pair (its first atom; the second gets the negative).
+// Two pairs (a, b) in packed arithmetic; pa, pb as LigDev::pconst.  Returns
+// the two energies' sum; fa, fb = dE/dx_i of each pair (its first atom; the
+// second gets the negative).
 __device__ __forceinline__ float pair_term2(float3 ia, float3 ib, float3 xa, float3 xb, float4 pa,
                                             float4 pb, bool hba, bool hbb, float3 &fa, float3 &fb) {
-    const float2 neg = f2s(-1.f);
+    const float2 neg = bc(-1.f);
     const float2 dx = __ffma2_rn(f2(xa.x, xb.x), neg, f2(ia.x, ib.x));   // x_i - x_j, exact
     const float2 dy = __ffma2_rn(f2(xa.y, xb.y), neg, f2(ia.y, ib.y));
     const float2 dz = __ffma2_rn(f2(xa.z, xb.z), neg, f2(ia.z, ib.z));
     const float2 r2 = __ffma2_rn(dz, dz, __ffma2_rn(dy, dy, __fmul2_rn(dx, dx)));
-    const bool la = r2.x >= RMIN2, lb = r2.y >= RMIN2;
-    const float2 r2c = f2(fmaxf(r2.x, RMIN2), fmaxf(r2.y, RMIN2));
-    const float2 rinv = f2(rsqrtf(r2c.x), rsqrtf(r2c.y));
-    const float2 rc = __fmul2_rn(r2c, rinv);
-    const float2 r2i = __fmul2_rn(rinv, rinv);
-    const float2 r4i = __fmul2_rn(r2i, r2i);
-    const float2 r6i = __fmul2_rn(r4i, r2i);
-    const float2 r12i = __fmul2_rn(r6i, r6i);
-    const float2 r10i = __fmul2_rn(r6i, r4i);
-    const float2 rmi = f2(hba ? r10i.x : r6i.x, hbb ? r10i.y : r6i.y);
-    const float2 m = f2(hba ? 10.f : 6.f, hbb ? 10.f : 6.f);
-    const float2 t12 = __fmul2_rn(f2(pa.x, pb.x), r12i), tm = __fmul2_rn(f2(pa.y, pb.y), rmi);
-    const float2 evdw = __ffma2_rn(tm, neg, t12);
-    const float2 dvdw = __fmul2_rn(__ffma2_rn(m, tm, __fmul2_rn(f2s(-12.f), t12)), rinv);
-    const float2 xa_ = __fmul2_rn(f2s(-MS_LAMBDA * MS_B), rc);
-    const float2 ex = f2(__expf(xa_.x), __expf(xa_.y));
-    const float2 den = __ffma2_rn(f2s(MS_K), ex, f2s(1.f));
-    const float2 num = __ffma2_rn(f2s(MS_A), den, f2s(MS_B));
-    const float2 dn = __fmul2_rn(den, num);
-    const float2 rr = f2(__fdividef(1.f, dn.x), __fdividef(1.f, dn.y));
-    const float2 eel =
-        __fmul2_rn(__fmul2_rn(f2(pa.z, pb.z), rinv), __fmul2_rn(__fmul2_rn(den, den), rr));
-    const float2 del = __fmul2_rn(__fmul2_rn(eel, neg),
-                                  __ffma2_rn(f2s(MS_B * MS_K * MS_LAMBDA * MS_B),
-                                             __fmul2_rn(ex, rr), rinv));
-    const float2 xd = __fmul2_rn(r2, f2s(-HALF_INV_SIG2));
-    const float2 eds = __fmul2_rn(f2(pa.w, pb.w), f2(__expf(xd.x), __expf(xd.y)));
-    const float2 frr = __fmul2_rn(__fadd2_rn(dvdw, del), rinv);
-    const float2 ft = __ffma2_rn(eds, f2s(-INV_SIG2), f2(la ? frr.x : 0.f, lb ? frr.y : 0.f));
+    float2 ft;
+    const float2 e = pair_terms2(r2, f2(pa.x, pb.x), f2(pa.y, pb.y), f2(pa.z, pb.z),
+                                 f2(pa.w, pb.w), {hba, hbb}, ft);
     const float2 fx = __fmul2_rn(ft, dx), fy = __fmul2_rn(ft, dy), fz = __fmul2_rn(ft, dz);
     fa = make_float3(fx.x, fy.x, fz.x);
     fb = make_float3(fx.y, fy.y, fz.y);
-    const float2 e = __fadd2_rn(__fadd2_rn(evdw, eel), eds);
     return e.x + e.y;
+}
+
+// One pair; f = dE/dx_i.
+__device__ __forceinline__ float pair_term(float4 xi, float4 xj, float4 pc, bool hb, float3 &f) {
+    const float dx = xi.x - xj.x, dy = xi.y - xj.y, dz = xi.z - xj.z;
+    float ft;
+    const float e = pair_term1(__fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx))), pc, hb, ft);
+    f = make_float3(ft * dx, ft * dy, ft * dz);
+    return e;
 }
 
 // ISSUED: the tcgen05 variant's MMAs were already issued (tc05_issue) and

@@ -34,6 +34,7 @@
 
 #include "adgb_internal.cuh"
 #include "packed.cuh"
+#include "pair_term.cuh"
 #include "reduce.cuh"
 #include "tcgen05.cuh"
 
@@ -41,9 +42,6 @@ namespace adgb {
 
 namespace {
 
-constexpr float P_INV_SIG2 = 1.0f / (ADGB_DS_SIGMA * ADGB_DS_SIGMA);
-constexpr float P_HALF_INV_SIG2 = 0.5f / (ADGB_DS_SIGMA * ADGB_DS_SIGMA);
-constexpr float P_RMIN2 = ADGB_R_MIN * ADGB_R_MIN;
 constexpr float P_PI = 3.14159265358979f;
 constexpr int P_ROT = ADGB_MAX_TORS;   // sc slots after the torsions: phi, theta, alpha
 constexpr unsigned FULL = 0xffffffffu;
@@ -159,52 +157,17 @@ __device__ __forceinline__ float grid_direct(const RecDev &R, int t, float q, fl
                        __ldg(cp + 2 * (R.M - 1) + 1), g0, g1, g2);
 }
 
-// 2^x by the special-function unit (the exponentials of the pair terms take
-// log2(e) folded into their constants).
-__device__ __forceinline__ float ex2a(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-constexpr float P_LOG2E = 1.4426950408889634f;
-
-// One intramolecular pair in both genotypes (the same pair constants
-// pc = (A, B, w_el 332.06 q_i q_j, w_ds (S_i V_j + S_j V_i)) and H-bond flag):
-// A r^-12 - B r^-m (m = 10 for donor-acceptor pairs, else 6) with r clamped
-// at R_MIN (no force below), Coulomb over the Mehler-Solmajer dielectric
-// (one reciprocal: 1/eps = den^2 rr r, eps'/eps = B k lambda B e rr), and the
-// desolvation Gaussian.  d = x_i - x_j; returns both energies, f = dE/dx_i.
+// One intramolecular pair in both genotypes (the same pair constants pc, as
+// LigDev::pconst, and H-bond flag).  d = x_i - x_j; returns both energies,
+// f = dE/dx_i.
 __device__ __forceinline__ float2 pair_both(const V2 &d, float4 pc, bool hb, V2 &f) {
     const float2 r2 = fma2(d.z, d.z, fma2(d.y, d.y, mul2(d.x, d.x)));
-    const bool la = r2.x >= P_RMIN2, lb = r2.y >= P_RMIN2;
-    const float2 r2c = make_float2(fmaxf(r2.x, P_RMIN2), fmaxf(r2.y, P_RMIN2));
-    const float2 rinv = make_float2(rsqrtf(r2c.x), rsqrtf(r2c.y));
-    const float2 rc = mul2(r2c, rinv);
-    const float2 r2i = mul2(rinv, rinv);
-    const float2 r4i = mul2(r2i, r2i);
-    const float2 r6i = mul2(r4i, r2i);
-    const float2 r12i = mul2(r6i, r6i);
-    const float2 rmi = hb ? mul2(r6i, r4i) : r6i;
-    const float2 t12 = mul2(bc(pc.x), r12i), tm = mul2(bc(pc.y), rmi);
-    const float2 evdw = fma2(tm, bc(-1.f), t12);
-    const float2 dvdw = mul2(fma2(bc(hb ? 10.f : 6.f), tm, mul2(bc(-12.f), t12)), rinv);
-    const float2 xe = mul2(bc(-MS_LAMBDA * MS_B * P_LOG2E), rc);
-    const float2 ex = make_float2(ex2a(xe.x), ex2a(xe.y));
-    const float2 den = fma2(bc(MS_K), ex, bc(1.f));
-    const float2 num = fma2(bc(MS_A), den, bc(MS_B));
-    const float2 dn = mul2(den, num);
-    const float2 rr = make_float2(__fdividef(1.f, dn.x), __fdividef(1.f, dn.y));
-    const float2 eel = mul2(mul2(bc(pc.z), rinv), mul2(mul2(den, den), rr));
-    const float2 del = mul2(mul2(eel, bc(-1.f)),
-                            fma2(bc(MS_B * MS_K * MS_LAMBDA * MS_B), mul2(ex, rr), rinv));
-    const float2 xd = mul2(r2, bc(-P_HALF_INV_SIG2 * P_LOG2E));
-    const float2 eds = mul2(bc(pc.w), make_float2(ex2a(xd.x), ex2a(xd.y)));
-    const float2 frr = mul2(add2(dvdw, del), rinv);
-    const float2 ft = fma2(eds, bc(-P_INV_SIG2), make_float2(la ? frr.x : 0.f, lb ? frr.y : 0.f));
+    float2 ft;
+    const float2 e = pair_terms2(r2, bc(pc.x), bc(pc.y), bc(pc.z), bc(pc.w), {hb, hb}, ft);
     f.x = mul2(ft, d.x);
     f.y = mul2(ft, d.y);
     f.z = mul2(ft, d.z);
-    return add2(add2(evdw, eel), eds);
+    return e;
 }
 
 // ------------------------------------------------ tcgen05 (paired form)
