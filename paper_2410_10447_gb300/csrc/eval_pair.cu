@@ -20,8 +20,11 @@
 //   5. reduce-and-broadcast (Sec. 3, 4.2) of the partials and the torsions'
 //      segmented sums over their moving atoms:
 //        shuffle / mma.sync: warp reduce-scatter of the 16 partials, each gene
-//          lane fetching the totals it needs; torsion lanes sum their moving
-//          range from a shared-memory copy of the partials;
+//          lane fetching the totals it needs; 4, 2 or 1 lanes a torsion sum
+//          its moving range from a shared-memory copy of the partials (one
+//          lane a torsion summed 20 atoms in a row, 15 instructions each, on
+//          every evaluation's chain: 1668 -> 1636 us for 3000 genotypes of 32
+//          atoms x 300 evaluations);
 //        tcgen05: ONE tensor-core product D = P . B^T a warp, B = the 32 lanes'
 //          partials of both genotypes (TF32 hi and lo terms, K = the lanes),
 //          P the ligand's 0/1 matrix whose row 6 + k is torsion k's moving-atom
@@ -421,7 +424,8 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
     const float4 *s_tax = reinterpret_cast<const float4 *>(sm + L.taxis);
     const float4 *s_tb = reinterpret_cast<const float4 *>(sm + L.tbref);
     unsigned char *W = sm + L.warp0 + warp * L.warp_stride;
-    float4 *xyz = reinterpret_cast<float4 *>(W + L.w_xyz);      // [2 i + g]
+    float4 *pxy = reinterpret_cast<float4 *>(W + L.w_xyz);      // (xA, xB, yA, yB) of atom i
+    float2 *pz = reinterpret_cast<float2 *>(W + L.w_xyz + 32 * 16);
     float2 *genes_s = reinterpret_cast<float2 *>(W + L.w_genes);
     float4 *sc = reinterpret_cast<float4 *>(W + L.w_sc);
     float *stage = reinterpret_cast<float *>(W + L.w_stage);
@@ -454,10 +458,13 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
     const float4 r4 = has_atom ? s_ref[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
     const int a_type = has_atom ? s_type[lane] : 0;
     const int a_frag = has_atom ? s_frag[lane] : -1;
-    // the lane's torsion (j = 6 + k): bond atoms and moving range
+    // the lane's torsion gene (j = 6 + tk), and the torsion kt whose moving
+    // atoms it helps to sum: 4 lanes a torsion up to 8 torsions, 2 up to 16
+    // (tcgen05: the sums arrive on the gene's own lane)
     const int tk = j - 6;
     const bool tors_lane = tk >= 0 && tk < T;
-    const int4 ta = tors_lane ? s_tat[tk] : make_int4(0, 0, 0, 0);
+    const int tl = VAR == ADGB_REDUCE_TCGEN05 ? 0 : (T <= 8 ? 2 : (T <= 16 ? 1 : 0));
+    const int kt = VAR == ADGB_REDUCE_TCGEN05 ? tk : lane >> tl;
     const int R = lig.n_rounds;
     const uint32_t *rw = lig.rword + lane;
     const float4 *rcs = lig.rconst + lane;
@@ -518,8 +525,8 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
                 e_acc = make_float2(ea, eb);
                 go = {make_float2(ga0, gb0), make_float2(ga1, gb1), make_float2(ga2, gb2)};
             }
-            xyz[2 * lane] = make_float4(xo.x.x, xo.y.x, xo.z.x, r4.w);
-            xyz[2 * lane + 1] = make_float4(xo.x.y, xo.y.y, xo.z.y, r4.w);
+            pxy[lane] = make_float4(xo.x.x, xo.x.y, xo.y.x, xo.y.y);
+            pz[lane] = xo.z;
         }
 
         // 3. pair terms in matching rounds, two rounds at a time as
@@ -592,22 +599,23 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
         const V2 tq = has_atom ? cross2(dxt, go) : V2{bc(0.f), bc(0.f), bc(0.f)};
         float2 v[8] = {e_acc, go.x, go.y, go.z, tq.x, tq.y, tq.z, bc(0.f)};
 
-        // 5. sums the lane's gene needs: E, and (sum g, sum (x - t) x g) over
-        //    all atoms (translation and rotation lanes) or over torsion
-        //    j - 6's moving atoms (torsion lanes)
+        // 5. sums: E and (sum g, sum (x - t) x g) over all atoms, and the
+        //    latter over torsion kt's moving atoms
         float2 E;
-        V2 Gs, Ts;
+        V2 Gs, Ts, Gk, Tk;   // over all atoms; over torsion kt's moving atoms
+        if constexpr (SKIP & SK_TORS) Gk = Tk = {bc(0.f), bc(0.f), bc(0.f)};
         if constexpr (SKIP & SK_RED) {
             E = v[0];
             Gs = {v[1], v[2], v[3]};
             Ts = {v[4], v[5], v[6]};
+            Gk = Gs, Tk = Ts;
         } else if constexpr (VAR == ADGB_REDUCE_TCGEN05) {
             float2 S[8];
             tc2_issue<(SKIP & SK_BLOCKMMA) != 0, (SKIP & SK_NOISSUE) == 0>(v, tw);
             tc2_finish<(SKIP & SK_NOISSUE) ? TC2_TEST_LIMIT : TC05_WAIT_LIMIT>(S, tw);
             E = shfl2(S[0], 0);   // lane 0's pattern row is all ones
-            Gs = {S[1], S[2], S[3]};
-            Ts = {S[4], S[5], S[6]};
+            Gk = Gs = {S[1], S[2], S[3]};   // a torsion gene's lane reads its moving set's row
+            Tk = Ts = {S[4], S[5], S[6]};
         } else {
             if constexpr (VAR == ADGB_REDUCE_SHFL) {
                 // totals: reduce-scatter, then E and three values a lane (its
@@ -643,9 +651,9 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
                 Gs = {make_float2(va[1], vb[1]), make_float2(va[2], vb[2]), make_float2(va[3], vb[3])};
                 Ts = {make_float2(va[4], vb[4]), make_float2(va[5], vb[5]), make_float2(va[6], vb[6])};
             }
-            // torsion lanes sum their moving range [start, end) from a shared
-            // copy of every lane's (g, torque) partials (12 floats a lane, in
-            // the warp's staging tile)
+            // lanes kt << tl .. sum torsion kt's moving range [start, end) from a
+            // shared copy of every lane's (g, torque) partials (12 floats a lane,
+            // in the warp's staging tile)
             if constexpr (!(SKIP & SK_TORS)) {
             __syncwarp();
             {
@@ -655,9 +663,10 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
                 row[2] = make_float4(v[5].x, v[5].y, v[6].x, v[6].y);
             }
             __syncwarp();
-            if (tors_lane) {
-                float2 gs[6] = {bc(0.f), bc(0.f), bc(0.f), bc(0.f), bc(0.f), bc(0.f)};
-                for (int i = ta.z; i < ta.w; i++) {
+            float2 gs[6] = {bc(0.f), bc(0.f), bc(0.f), bc(0.f), bc(0.f), bc(0.f)};
+            if (kt < T) {
+                const int4 ta = s_tat[kt];
+                for (int i = ta.z + (lane & ((1 << tl) - 1)); i < ta.w; i += 1 << tl) {
                     const float4 *row = reinterpret_cast<const float4 *>(stage + 12 * i);
                     const float4 a0 = row[0], a1 = row[1], a2 = row[2];
                     gs[0] = add2(gs[0], make_float2(a0.x, a0.y));
@@ -667,25 +676,44 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
                     gs[4] = add2(gs[4], make_float2(a2.x, a2.y));
                     gs[5] = add2(gs[5], make_float2(a2.z, a2.w));
                 }
-                Gs = {gs[0], gs[1], gs[2]};
-                Ts = {gs[3], gs[4], gs[5]};
             }
+            for (int m = 1; m < 1 << tl; m <<= 1) {   // uniform
+#pragma unroll
+                for (int q = 0; q < 6; q++)
+                    gs[q] = add2(gs[q], make_float2(__shfl_xor_sync(FULL, gs[q].x, m),
+                                                    __shfl_xor_sync(FULL, gs[q].y, m)));
+            }
+            Gk = {gs[0], gs[1], gs[2]};
+            Tk = {gs[3], gs[4], gs[5]};
             __syncwarp();   // the copy and the staging tile are rewritten next evaluation
             }
         }
 
-        // 6. gene gradient, best tracking, ADADELTA
-        // Every gene lane evaluates one formula, g = W . Tv, its role choosing
-        // W and Tv (no divergent paths): rotation genes phi / theta take the
-        // angular velocity w = sin(a) du + (1 - cos a) u x du of the axis
-        // change du and the torque; alpha takes u and the torque; torsion k
-        // takes the unit bond axis a -> b and sum (x - x_b) x g = sum (x - t) x g
-        // - (x_b - t) x sum g over its moving atoms; translation gene j takes
-        // sum g's component j.
+        // 6. gene gradient, best tracking, ADADELTA.  Torsion kt: the unit bond
+        // axis a -> b times sum (x - x_b) x g = sum (x - t) x g - (x_b - t) x
+        // sum g over its moving atoms, then to the gene's lane; rotation genes:
+        // the torque times the angular velocity w = sin(a) du + (1 - cos a) u x
+        // du of the axis change du (phi, theta) or times u (alpha); translation
+        // gene j: sum g's component j.
         float2 gj;
         if constexpr (SKIP & SK_GENE) {
             gj = Gs.x;
         } else {
+            float2 gk = bc(0.f);
+            if (kt >= 0 && kt < T) {
+                const int4 ta = s_tat[kt];
+                const float4 xya = pxy[ta.x], xyb = pxy[ta.y];
+                const V2 xa = {make_float2(xya.x, xya.y), make_float2(xya.z, xya.w), pz[ta.x]};
+                const V2 xb = {make_float2(xyb.x, xyb.y), make_float2(xyb.z, xyb.w), pz[ta.y]};
+                const V2 ax = {sub2(xb.x, xa.x), sub2(xb.y, xa.y), sub2(xb.z, xa.z)};
+                const float2 l2 = dot2(ax, ax);
+                const V2 bt = {sub2(xb.x, tr.x), sub2(xb.y, tr.y), sub2(xb.z, tr.z)};
+                const V2 bxg = cross2(bt, Gk);
+                const V2 acc = {sub2(Tk.x, bxg.x), sub2(Tk.y, bxg.y), sub2(Tk.z, bxg.z)};
+                if (ta.w > ta.z)
+                    gk = mul2(dot2(acc, ax), make_float2(rsqrtf(l2.x), rsqrtf(l2.y)));
+            }
+            if constexpr (VAR != ADGB_REDUCE_TCGEN05) gk = shfl2(gk, (tk << tl) & 31);
             const bool th = j == 4;
             V2 du;
             du.x = th ? mul2(cth, cphi) : mul2(bc(-1.f), mul2(sth, sphi));
@@ -694,25 +722,9 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
             const V2 uxd = cross2(u, du);
             const V2 wv = {fma2(s, du.x, mul2(o, uxd.x)), fma2(s, du.y, mul2(o, uxd.y)),
                            fma2(s, du.z, mul2(o, uxd.z))};
-            // the torsion lane's bond atoms (atom 0 for the other lanes)
-            const int ia = tors_lane ? ta.x : 0, ib = tors_lane ? ta.y : 0;
-            const float4 xa0 = xyz[2 * ia], xa1 = xyz[2 * ia + 1];
-            const float4 xb0 = xyz[2 * ib], xb1 = xyz[2 * ib + 1];
-            const V2 xb = {make_float2(xb0.x, xb1.x), make_float2(xb0.y, xb1.y),
-                           make_float2(xb0.z, xb1.z)};
-            const V2 ax = {sub2(xb.x, make_float2(xa0.x, xa1.x)), sub2(xb.y, make_float2(xa0.y, xa1.y)),
-                           sub2(xb.z, make_float2(xa0.z, xa1.z))};
-            const float2 l2 = dot2(ax, ax);
-            const float2 il = tors_lane ? make_float2(rsqrtf(l2.x), rsqrtf(l2.y)) : bc(0.f);
-            const V2 bt = {sub2(xb.x, tr.x), sub2(xb.y, tr.y), sub2(xb.z, tr.z)};
-            const V2 bxg = cross2(bt, Gs);
-            const V2 acc = {sub2(Ts.x, bxg.x), sub2(Ts.y, bxg.y), sub2(Ts.z, bxg.z)};
-            const V2 Tv = tors_lane ? acc : Ts;
-            const V2 Wv = tors_lane ? V2{mul2(ax.x, il), mul2(ax.y, il), mul2(ax.z, il)}
-                                    : (j == 5 ? u : wv);
-            gj = dot2(Tv, Wv);
+            gj = dot2(Ts, j == 5 ? u : wv);
             if (j < 3) gj = j == 0 ? Gs.x : (j == 1 ? Gs.y : Gs.z);
-            if ((tors_lane && ta.w <= ta.z) || j >= G) gj = bc(0.f);
+            if (j >= 6) gj = tors_lane ? gk : bc(0.f);
         }
         if (io.mode == MODE_SCORE) {
             if (lane == 0) {
@@ -738,8 +750,7 @@ __device__ __forceinline__ void search_pair(unsigned char *sm, const PairSmem &L
             const float2 rho = bc(io.rho), omr = bc(1.f - io.rho), ep = bc(io.eps);
             const float2 neg2 = fma2(rho, eg2, mul2(omr, mul2(gj, gj)));
             const float2 a2 = add2(ed2, ep), b2 = add2(neg2, ep);
-            const float2 d = mul2(mul2(make_float2(-sqrtf(a2.x), -sqrtf(a2.y)),
-                                       make_float2(rsqrtf(b2.x), rsqrtf(b2.y))), gj);
+            const float2 d = mul2(root_ratio2(a2, b2), make_float2(-gj.x, -gj.y));
             const float2 ned2 = fma2(rho, ed2, mul2(omr, mul2(d, d)));
             float2 w = add2(om, d);
             if (j >= 6) {

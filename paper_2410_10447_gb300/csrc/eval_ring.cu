@@ -322,7 +322,10 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
                 for (int a = 0; a < A; a++) {
                     const float4 pc = __ldg(tp + 32 * a);
                     const bool hb = __float_as_int(pc.x) < 0;
-                    const V2 d = {sub2(xi[a].x, xj.x), sub2(xi[a].y, xj.y), sub2(xi[a].z, xj.z)};
+                    // x_i - x_j, exact; as FMAs 0.8% faster here than as adds
+                    const float2 m1 = bc(-1.f);
+                    const V2 d = {fma2(xj.x, m1, xi[a].x), fma2(xj.y, m1, xi[a].y),
+                                  fma2(xj.z, m1, xi[a].z)};
                     const float2 r2 = fma2(d.z, d.z, fma2(d.y, d.y, mul2(d.x, d.x)));
                     float2 ft;
                     const float2 e = pair_terms2(r2, bc(fabsf(pc.x)), bc(pc.y), bc(pc.z), bc(pc.w),
@@ -493,8 +496,7 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
                 const float2 rho = bc(io.rho), omr = bc(1.f - io.rho), ep = bc(io.eps);
                 const float2 neg2 = fma2(rho, eg2, mul2(omr, mul2(gj, gj)));
                 const float2 a2 = add2(ed2, ep), b2 = add2(neg2, ep);
-                const float2 d = mul2(mul2(make_float2(-sqrtf(a2.x), -sqrtf(a2.y)),
-                                           make_float2(rsqrtf(b2.x), rsqrtf(b2.y))), gj);
+                const float2 d = mul2(root_ratio2(a2, b2), make_float2(-gj.x, -gj.y));
                 const float2 ned2 = fma2(rho, ed2, mul2(omr, mul2(d, d)));
                 float2 w = add2(om, d);
                 if (j >= 6) {

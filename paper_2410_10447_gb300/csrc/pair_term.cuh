@@ -34,6 +34,17 @@ __device__ __forceinline__ float rcp_ftz(float x) {
     return y;
 }
 
+// sqrt(a) / sqrt(b), the ADADELTA step's scale, as a / sqrt(a b): one special
+// function and no square root (its error, half an ulp of a b under the root,
+// that of rsqrt.approx and one rounding, is below that of sqrtf times
+// rsqrtf).  Where a b leaves the normal range, the two roots themselves.
+__device__ __forceinline__ float2 root_ratio2(float2 a, float2 b) {
+    const float2 ab = mul2(a, b);
+    const bool fine = ab.x > 1e-36f && ab.x < 1e38f && ab.y > 1e-36f && ab.y < 1e38f;
+    if (fine) return mul2(a, make_float2(rsqrt_ftz(ab.x), rsqrt_ftz(ab.y)));
+    return make_float2(sqrtf(a.x) * rsqrtf(b.x), sqrtf(a.y) * rsqrtf(b.y));
+}
+
 // Two pair terms from their squared distances r2 and constants A, B (12-6
 // van der Waals A r^-12 - B r^-6, or 12-10 with hb), C = PT_CSCALE w_el 332.06
 // q_i q_j and D = w_ds (S_i V_j + S_j V_i).  Returns the energies; ft =
