@@ -222,8 +222,13 @@ def _ptr(x):
 
 
 def _stream():
+    """Raw pointer of torch's current stream (without a Stream object where
+    torch has the call for it: a scoring call of a few poses takes 10 us)."""
     import torch
-    return torch.cuda.current_stream().cuda_stream
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _f32(a):

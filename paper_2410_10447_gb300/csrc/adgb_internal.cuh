@@ -4,6 +4,9 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+#include <atomic>
+
 #include "adgb.h"  // include/ is on the include path
 
 namespace adgb {
@@ -330,25 +333,40 @@ struct EvalCfg {
 // -> 74%; on the one-genotype and Solis-Wets kernels 1-2% slower, so they
 // keep the default).  The tcgen05 form keeps the default too (no gain
 // measured: its P and B operands take 30 KB a block).
-template <typename K>
-inline cudaError_t prefer_l1(K k, int smem, int threads) {
-    int dev = 0, per_sm = 0, reserved = 0, regs_sm = 0;
-    cudaFuncAttributes fa;
+// The hint is a property of the kernel on its device, so it is set when it
+// differs from the last one set for this kernel (a scoring call of a few poses
+// takes about 10 us in all, and the six queries and the set took 2 of them).
+template <auto K>
+inline void prefer_l1(int smem, int threads) {
+    static std::atomic<uint64_t> last{0};
+    int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
+    const uint64_t key = (uint64_t)(dev + 1) << 48 | (uint64_t)threads << 32 | (uint32_t)smem;
+    if (e == cudaSuccess && last.load(std::memory_order_relaxed) == key) return;
+    int per_sm = 0, reserved = 0, regs_sm = 0;
+    cudaFuncAttributes fa;
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
-    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, K);
     if (e == cudaSuccess && per_sm > 0) {
         const int regs_block = ((fa.numRegs * 32 + 255) / 256) * 256 * (threads / 32);
-        const int blocks = regs_block > 0 ? max(1, regs_sm / regs_block) : 1;
+        const int blocks = regs_block > 0 ? std::max(1, regs_sm / regs_block) : 1;
         const long need = (long)blocks * (smem + (long)fa.sharedSizeBytes + reserved);
-        const int pct = (int)max(1L, min(100L, (need * 100 + per_sm - 1) / per_sm));
-        e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
+        const int pct = (int)std::max(1L, std::min(100L, (need * 100 + per_sm - 1) / per_sm));
+        e = cudaFuncSetAttribute(K, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
     }
     // a hint: a refusal leaves the default carveout and is not the launch's error
-    if (e != cudaSuccess) (void)cudaGetLastError();
-    return cudaSuccess;
+    if (e == cudaSuccess) last.store(key, std::memory_order_relaxed);
+    else (void)cudaGetLastError();
+}
+
+// Dynamic shared memory a launch may take without asking for more.
+constexpr int SMEM_DEFAULT_LIMIT = 46 * 1024;   // of 48 KB, static shared memory included
+template <typename K>
+inline cudaError_t allow_smem(K k, int smem) {
+    if (smem <= SMEM_DEFAULT_LIMIT) return cudaSuccess;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
 }
 
 // Host-side launchers (eval.cu, reduce_bench.cu).

@@ -1025,7 +1025,7 @@ int eval_smem_bytes(int layout_bytes, const EvalCfg &cfg, int device, bool items
 template <int TPP, int VAR>
 static cudaError_t launch_items_t(const ItemsArgs &a, int smem, int grid, cudaStream_t s) {
     auto k = eval_items_kernel<TPP, VAR>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     k<<<grid, TPP * a.ppb, smem, s>>>(a);
     return cudaGetLastError();
@@ -1134,7 +1134,7 @@ static cudaError_t launch_t(const EvalArgs &a, int ppb, int smem, cudaStream_t s
     constexpr int NG_MAX = (MAX_GENES + TPP - 1) / TPP;
     auto k = (NG_MAX > 1 && 6 + a.lig.n_tors <= TPP) ? eval_kernel<TPP, VAR, 1>
                                                       : eval_kernel<TPP, VAR, NG_MAX>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     const int blocks = (a.n + ppb - 1) / ppb;
     k<<<blocks, TPP * ppb, smem, s>>>(a);
@@ -1199,7 +1199,7 @@ cudaError_t launch_eval(const RecDev &rec, const LigDev &lig, const EvalCfg &cfg
 template <int TPP, int VAR>
 static cudaError_t launch_sw_t(const SwArgs &a, int ppb, int smem, cudaStream_t s) {
     auto k = sw_kernel<TPP, VAR>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     k<<<(a.n + ppb - 1) / ppb, TPP * ppb, smem, s>>>(a);
     return cudaGetLastError();

@@ -937,9 +937,10 @@ cudaError_t pair_items_occupancy(int threads, int smem, int device, int *per_sm)
 template <int VAR>
 cudaError_t launch_pair_items_t(const PairItemsArgs &a, int smem, int grid, cudaStream_t s) {
     auto k = eval_pair_items_kernel<VAR>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess && VAR != ADGB_REDUCE_TCGEN05) e = prefer_l1(k, smem, 32 * ((a.ppb + 1) / 2));
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05)
+        prefer_l1<eval_pair_items_kernel<VAR>>(smem, 32 * ((a.ppb + 1) / 2));
     k<<<grid, 32 * ((a.ppb + 1) / 2), smem, s>>>(a);
     return cudaGetLastError();
 }
@@ -1019,9 +1020,9 @@ template <int VAR, int SKIP = 0>
 static cudaError_t launch_pair_t(const PairArgs &a, int smem, cudaStream_t s) {
     auto k = eval_pair_kernel<VAR, SKIP>;
     const int warps = (a.ppb + 1) / 2;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess && VAR != ADGB_REDUCE_TCGEN05) e = prefer_l1(k, smem, 32 * warps);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) prefer_l1<eval_pair_kernel<VAR, SKIP>>(smem, 32 * warps);
     k<<<(a.n + a.ppb - 1) / a.ppb, 32 * warps, smem, s>>>(a);
     return cudaGetLastError();
 }

@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(128, 4) eval_ring_items_kernel(const WorkItem 
 template <int A, int VAR, int MB>
 cudaError_t launch_ring_t(const RingArgs &a, int threads, int smem, cudaStream_t s) {
     auto k = eval_ring_kernel<A, VAR, MB>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     k<<<(a.n + 1) / 2, threads, smem, s>>>(a);
     return cudaGetLastError();
@@ -641,7 +641,7 @@ template <int A, int VAR>
 cudaError_t launch_ring_items_t(const WorkItem *items, int n_items, const LigDev *ligs,
                                 const RecDev *recs, int threads, int smem, cudaStream_t s) {
     auto k = eval_ring_items_kernel<A, VAR>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     k<<<n_items, threads, smem, s>>>(items, ligs, recs);
     return cudaGetLastError();
