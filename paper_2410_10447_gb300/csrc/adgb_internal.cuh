@@ -239,25 +239,43 @@ struct RingShape {
     int pos_len;          // positions the sweep reads (the ring and its continuation)
     int copy_len, copies; // entries of a force copy (index: ring atom minus the slice's first
                           // step), and copies: one a team, or one a warp with windows
+    int pos_res, copy_res; // a = 4: entries a residue class (ring_index)
 };
-// a = 3 or 5 (odd: no bank conflicts), whichever leaves fewer idle lanes at
-// N atoms; 4 warps (3 where the lanes span three windows).
+// a = 3, 4 or 5, whichever leaves the fewest idle lanes at N atoms (256 atoms:
+// 64 lanes of 4; with 3 a lane 86 of 96 lanes, with 5 52 of 64).
 __host__ __device__ inline RingShape ring_shape(int N) {
     RingShape r;
-    r.a = N <= 48 ? 3 : (N <= 80 ? 5 : (N <= 96 ? 3 : (N <= 160 ? 5 : 3)));
+    r.a = N <= 48 ? 3 : N <= 64 ? 4 : N <= 80 ? 5 : N <= 96 ? 3 : N <= 128 ? 4 : N <= 160 ? 5
+          : N <= 192 ? 3 : 4;
     r.la = (N + r.a - 1) / r.a;
     r.np = r.a * r.la;
     r.windows = (r.la + 31) / 32;
     r.teams = r.windows > 1 ? 1 : 32 / r.la;
-    r.warps = r.windows == 3 ? 3 : 4;
+    r.warps = 4;
     r.slices = r.windows > 1 ? r.warps / r.windows : r.teams * r.warps;
     const int s = r.np / 2 + r.a - 1;
     r.steps = (s + r.slices - 1) / r.slices;
     r.pos_len = r.a * (r.la - 1) + r.slices * r.steps + 1;
     r.copy_len = r.steps > r.a ? r.np - r.a + r.steps : r.np;
     r.copies = r.windows > 1 ? r.warps : r.teams * r.warps;
+    r.pos_res = r.a == 4 ? (r.pos_len + 3) / 4 : 0;
+    r.copy_res = r.a == 4 ? (r.copy_len + 3) / 4 : 0;
     return r;
 }
+// Where entry j of a position or force array lies.  Lanes a apart in j read
+// together: for odd a the 16-byte entries of 8 neighbouring lanes fall into
+// different bank groups as they are; for a = 4 the entries of each residue
+// class j mod 4 are contiguous (res of them).
+template <int A>
+__host__ __device__ inline int ring_index(int j, int res) {
+    return A == 4 ? (j & 3) * res + (j >> 2) : j;
+}
+// From entry j to j + 1.
+template <int A>
+__host__ __device__ inline int ring_next(int j, int res) {
+    return A == 4 ? ((j & 3) == 3 ? 1 - 3 * res : res) : 1;
+}
+__host__ __device__ inline int ring_entries(int len, int res) { return res ? 4 * res : len; }
 // Slice of the steps whose reactions copy c holds.
 __host__ __device__ inline int ring_slice(const RingShape &r, int c) {
     return r.windows > 1 ? c / r.windows : c;

@@ -63,8 +63,8 @@ struct Batch {
 };
 }  // namespace
 
-// Kinds of launches a batch may need: one a class of ring shapes (a = 3 or 5
-// with 4 warps, a = 3 with 3), two genotypes a warp, one genotype a warp.
+// Kinds of launches a batch may need: one a class of ring shapes (a = 3, 4 or
+// 5), two genotypes a warp, one genotype a warp.
 constexpr int BATCH_CLASSES = 5;
 
 struct adgb_ctx {

@@ -1,6 +1,6 @@
 // Fused scoring / ADADELTA local search of ligands of more than 32 atoms
-// (Sec. 2.1, Sec. 3; Table 1's gpu_gradient_minAD): one block of 3 or 4
-// warps searches two genotypes, packed (genotype A in .x, B in .y), so that
+// (Sec. 2.1, Sec. 3; Table 1's gpu_gradient_minAD): one block of 4 warps
+// searches two genotypes, packed (genotype A in .x, B in .y), so that
 // the ligand's pair constants, torsion tree and addresses are read and
 // computed once for both.
 //
@@ -9,8 +9,8 @@
 // j = A lane + s of the ring, computing its A pairs with it.  In a step every
 // lane's j is another atom, so the reaction on j is added to the warp's own
 // copy of the forces in shared memory without atomics: two loads, two stores
-// and a warp barrier for A pairs of two genotypes.  A odd puts a quarter
-// warp's 16-byte accesses into different banks without padding.  The steps
+// and a warp barrier for A pairs of two genotypes, all of them free of bank
+// conflicts (ring_index).  The steps
 // are split over the block's warps (and, for small ligands, over two or three
 // teams of lanes in a warp); every atom's owner then sums the copies.  The
 // pair constants come from a table in the order of the sweep (coalesced
@@ -26,9 +26,11 @@
 // or 128-thread group, forces through per-pair slots in shared memory) had its
 // LSU data pipe 73% busy at 256 atoms, 46% of the shared-memory wavefronts
 // bank-conflict replays, at 107K warp instructions an evaluation; this one
-// issues 45K.  Local search, M evaluations/s before -> with the sweep:
-// 45 atoms x 1000 genotypes 95 -> 156, 90 x 1500 31 -> 84, 128 x 8000
-// 17 -> 41, 192 x 6000 10 -> 27, 256 x 2048 6.2 -> 12.0, x 8192 6.8 -> 14.
+// issues 42K.  Local search, M evaluations/s before -> with the sweep:
+// 45 atoms x 1000 genotypes 95 -> 159, 64 x 8000 58 -> 121, 90 x 1500
+// 31 -> 85, 128 x 8000 17 -> 52, 192 x 6000 10 -> 28, 256 x 2048 6.2 -> 13.4,
+// x 8192 6.8 -> 15.5 (with 3 or 5 atoms a lane only, no 4: 64 x 8000 113,
+// 128 x 8000 43, 256 x 2048 12.1: idle lanes).
 //
 // Per evaluation (block barriers between the steps):
 //   1. gene threads publish genes and sin / (1 - cos) of every angle;
@@ -78,10 +80,11 @@ struct RingSmem {
         tatoms = o;  o = al16(o + 16 * Tn);
         taxis = o;   o = al16(o + 16 * Tn);
         tbref = o;   o = al16(o + 16 * Tn);
-        pxy = o;     o = al16(o + 16 * r.pos_len);
-        pz = o;      o = al16(o + 8 * r.pos_len);
-        cxy = o;     o = al16(o + 16 * r.copies * r.copy_len);
-        cz = o;      o = al16(o + 8 * r.copies * r.copy_len);
+        const int pe = ring_entries(r.pos_len, r.pos_res), ce = ring_entries(r.copy_len, r.copy_res);
+        pxy = o;     o = al16(o + 16 * pe);
+        pz = o;      o = al16(o + 8 * pe);
+        cxy = o;     o = al16(o + 16 * r.copies * ce);
+        cz = o;      o = al16(o + 8 * r.copies * ce);
         gxy = o;     o = al16(o + 16 * N);
         gz = o;      o = al16(o + 8 * N);
         genes = o;   o = al16(o + 8 * MAX_GENES);
@@ -215,8 +218,10 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
     float2 best_e = bc(INFINITY);
     // the lane's place in the ring sweep
     const RingLane rl = ring_lane(rs, warp, lane);
-    const int copy0 = rl.copy * rs.copy_len + A * rl.l;   // slot of step 0 in the lane's copy
-    const int pos0 = A * rl.l + rl.s0;
+    const int copy_ent = ring_entries(rs.copy_len, rs.copy_res);
+    const int copy0 = rl.copy * copy_ent;   // the lane's copy
+    auto pos_at = [&](int q) { return ring_index<A>(q, rs.pos_res); };
+    auto copy_at = [&](int q) { return ring_index<A>(q, rs.copy_res); };
     const float4 *table = lig.ring + (size_t)warp * rs.steps * A * 32 + lane;
     // the thread's genotype in steps 2 and 5 (blockDim.x is even)
     const int gen = t & 1;
@@ -268,7 +273,8 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
                 x.y = p.y + (m10 * p.x + m11 * p.y + m12 * p.z) + tr.y;
                 x.z = p.z + (m20 * p.x + m21 * p.y + m22 * p.z) + tr.z;
                 float *xyf = reinterpret_cast<float *>(pxy), *zf = reinterpret_cast<float *>(pz);
-                auto put = [&](int q) {
+                auto put = [&](int e) {
+                    const int q = pos_at(e);
                     xyf[4 * q + gen] = x.x;
                     xyf[4 * q + 2 + gen] = x.y;
                     zf[2 * q + gen] = x.z;
@@ -297,8 +303,8 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
             if ((lane & 2) == 0) red[16 * warp + 8 * gen + (lane >> 2)] = mine;
         }
         // the warp's copies of the forces start from zero
-        for (int q = lane; q < rs.teams * rs.copy_len; q += 32) {
-            const int c = warp * rs.teams * rs.copy_len + q;
+        for (int q = lane; q < rs.teams * copy_ent; q += 32) {
+            const int c = warp * rs.teams * copy_ent + q;
             cxy[c] = make_float4(0.f, 0.f, 0.f, 0.f);
             cz[c] = bc(0.f);
         }
@@ -310,13 +316,16 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
             V2 xi[A], fi[A];
 #pragma unroll
             for (int a = 0; a < A; a++) {
-                xi[a] = load_v2(pxy, pz, A * rl.l + a);
+                xi[a] = load_v2(pxy, pz, pos_at(A * rl.l + a));
                 fi[a] = {bc(0.f), bc(0.f), bc(0.f)};
             }
             const float4 *tp = table;
+            // atom a l + s0 + st of the ring and its place in the copy
+            int pj = pos_at(A * rl.l + rl.s0), cj = copy0 + copy_at(A * rl.l);
 #pragma unroll 2
             for (int st = 0; st < rs.steps; st++, tp += A * 32) {
-                const V2 xj = load_v2(pxy, pz, pos0 + st);
+                const V2 xj = load_v2(pxy, pz, A == 4 ? pj : pj + st);
+                if constexpr (A == 4) pj += ring_next<A>(rl.s0 + st, rs.pos_res);
                 V2 fj = {bc(0.f), bc(0.f), bc(0.f)};
 #pragma unroll
                 for (int a = 0; a < A; a++) {
@@ -334,12 +343,14 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
                     fi[a] = {fma2(ft, d.x, fi[a].x), fma2(ft, d.y, fi[a].y), fma2(ft, d.z, fi[a].z)};
                     fj = {fma2(ft, d.x, fj.x), fma2(ft, d.y, fj.y), fma2(ft, d.z, fj.z)};
                 }
-                const V2 c = load_v2(cxy, cz, copy0 + st);
+                const int ce = A == 4 ? cj : cj + st;
+                const V2 c = load_v2(cxy, cz, ce);
                 if (rl.active) {
                     const V2 n = {sub2(c.x, fj.x), sub2(c.y, fj.y), sub2(c.z, fj.z)};
-                    cxy[copy0 + st] = make_float4(n.x.x, n.x.y, n.y.x, n.y.y);
-                    cz[copy0 + st] = n.z;
+                    cxy[ce] = make_float4(n.x.x, n.x.y, n.y.x, n.y.y);
+                    cz[ce] = n.z;
                 }
+                if constexpr (A == 4) cj += ring_next<A>(st, rs.copy_res);
                 __syncwarp();   // the next step's slots were other lanes' in this one
             }
             // the lane's own atoms: slot of atom i is i - s0 around the ring
@@ -347,7 +358,7 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
             for (int a = 0; a < A; a++) {
                 int q = A * rl.l + a - rl.s0;
                 if (q < 0) q += rs.np;
-                q += rl.copy * rs.copy_len;
+                q = copy0 + copy_at(q);
                 if (rl.active) {
                     const V2 c = load_v2(cxy, cz, q);
                     const V2 n = {add2(c.x, fi[a].x), add2(c.y, fi[a].y), add2(c.z, fi[a].z)};
@@ -366,10 +377,10 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
                 for (int c = 0; c < rs.copies; c++) {
                     int q = i - 1 - ring_slice(rs, c) * rs.steps;
                     if (q < 0) q += rs.np;
-                    const V2 f = load_v2(cxy, cz, c * rs.copy_len + q);
+                    const V2 f = load_v2(cxy, cz, c * copy_ent + copy_at(q));
                     g = {add2(g.x, f.x), add2(g.y, f.y), add2(g.z, f.z)};
                     if (q + rs.np < rs.copy_len) {   // at most one more turn (copy_len < 2 np)
-                        const V2 h = load_v2(cxy, cz, c * rs.copy_len + q + rs.np);
+                        const V2 h = load_v2(cxy, cz, c * copy_ent + copy_at(q + rs.np));
                         g = {add2(g.x, h.x), add2(g.y, h.y), add2(g.z, h.z)};
                     }
                 }
@@ -388,9 +399,9 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
             V2 xb = acc;
             if (k < T) {
                 ta = s_tat[k];
-                xb = load_v2(pxy, pz, ta.y);
+                xb = load_v2(pxy, pz, pos_at(ta.y));
                 for (int i = ta.z + (t & 7); i < ta.w; i += 8) {
-                    const V2 g = load_v2(gxy, gz, i), x = load_v2(pxy, pz, i);
+                    const V2 g = load_v2(gxy, gz, i), x = load_v2(pxy, pz, pos_at(i));
                     const V2 d = {sub2(x.x, xb.x), sub2(x.y, xb.y), sub2(x.z, xb.z)};
                     const V2 c = cross2(d, g);
                     acc = {add2(acc.x, c.x), add2(acc.y, c.y), add2(acc.z, c.z)};
@@ -408,7 +419,7 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
             if (k < T && (t & 7) == 0) {
                 float2 gk = bc(0.f);
                 if (ta.w > ta.z) {
-                    const V2 xa = load_v2(pxy, pz, ta.x);
+                    const V2 xa = load_v2(pxy, pz, pos_at(ta.x));
                     const V2 ax = {sub2(xb.x, xa.x), sub2(xb.y, xa.y), sub2(xb.z, xa.z)};
                     const float2 l2 = dot2(ax, ax);
                     gk = mul2(dot2(ax, acc), make_float2(rsqrtf(l2.x), rsqrtf(l2.y)));
@@ -682,6 +693,7 @@ cudaError_t launch_eval_ring_items(const WorkItem *items, int n_items, const Lig
     const int smem = tc_smem_bytes(layout_bytes, warps, variant, dev);
     if (smem < 0) return cudaErrorInvalidValue;
     if (a == 3) return launch_ring_items_v<3>(items, n_items, ligs, recs, variant, 32 * warps, smem, s);
+    if (a == 4) return launch_ring_items_v<4>(items, n_items, ligs, recs, variant, 32 * warps, smem, s);
     return launch_ring_items_v<5>(items, n_items, ligs, recs, variant, 32 * warps, smem, s);
 }
 
@@ -713,6 +725,7 @@ cudaError_t launch_eval_ring(const RecDev &rec, const LigDev &lig, const EvalCfg
     const int smem = tc_smem_bytes(a.L.total, rs.warps, cfg.variant, dev);
     if (smem < 0) return cudaErrorInvalidValue;
     if (rs.a == 5) return launch_ring_v<5, 4>(a, cfg.variant, 32 * rs.warps, smem, s);
+    if (rs.a == 4) return launch_ring_v<4, 4>(a, cfg.variant, 32 * rs.warps, smem, s);
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
