@@ -744,6 +744,7 @@ __device__ __forceinline__ void search_pose_sw(unsigned char *sm, const SmemLayo
         const float m01 = o * u.x * u.y - s * u.z, m10 = o * u.x * u.y + s * u.z;
         const float m02 = o * u.x * u.z + s * u.y, m20 = o * u.x * u.z - s * u.y;
         const float m12 = o * u.y * u.z - s * u.x, m21 = o * u.y * u.z + s * u.x;
+        float3 xo = make_float3(0.f, 0.f, 0.f);   // the lane's atom (one warp)
         float e_part = 0.f;
         for (int i = gt; i < N; i += TPP) {
             const float4 r4 = s_ref[i];
@@ -754,29 +755,75 @@ __device__ __forceinline__ void search_pose_sw(unsigned char *sm, const SmemLayo
             x.y = p.y + (m10 * p.x + m11 * p.y + m12 * p.z) + tr.y;
             x.z = p.z + (m20 * p.x + m21 * p.y + m22 * p.z) + tr.z;
             xyz[i] = make_float4(x.x, x.y, x.z, r4.w);
+            xo = x;
             float3 gi;
             e_part += inter_atom(rec, s_type[i], r4.w, x, gi);
         }
-        group_sync<TPP>(group);
-        int p = gt;
-        for (; p + TPP < NP; p += 2 * TPP) {  // pairs p and p + TPP, packed arithmetic
-            const uint32_t pa = prs[p], pb = prs[p + TPP];
+        if (TPP == 32 && lig.r_lanes == 32 && lig.n_rounds > 0 && 64 * lig.n_rounds <= 3 * NP) {
+            // matching rounds, two at a time: the partner's position by shuffles
+            // and coalesced constants (from the pair list, four 16-byte loads of
+            // random atoms for two pairs kept the LSU data pipe 70% busy).  Where
+            // two thirds of the rounds' lanes have a pair: 32 atoms (364 pairs,
+            // 11 rounds) 266 -> 242 us for 3000 genotypes x 60 evaluations, 24
+            // (186, 8) 206 -> 199; 16 (57, 5), the other side, 157 -> 169.
+            const uint32_t *rw = lig.rword + gt;
+            const float4 *rc = lig.rconst + gt;
+            auto partner = [&](uint32_t w) {
+                const int pj = w & 31;
+                return make_float3(__shfl_sync(0xffffffffu, xo.x, pj),
+                                   __shfl_sync(0xffffffffu, xo.y, pj),
+                                   __shfl_sync(0xffffffffu, xo.z, pj));
+            };
+            int r = 0;
             float3 fa, fb;
-            e_part += pair_term2(xyz3(xyz[pa & 255]), xyz3(xyz[pb & 255]),
-                                 xyz3(xyz[(pa >> 8) & 255]), xyz3(xyz[(pb >> 8) & 255]),
-                                 __ldg(pconst + p), __ldg(pconst + p + TPP), (pa >> 24) & 1,
-                                 (pb >> 24) & 1, fa, fb);
+#pragma unroll 2
+            for (; r + 1 < lig.n_rounds; r += 2) {
+                const uint32_t wa = __ldg(rw + 32 * r), wb = __ldg(rw + 32 * (r + 1));
+                const float4 pa = __ldg(rc + 32 * r), pb = __ldg(rc + 32 * (r + 1));
+                const float3 xa = partner(wa), xb = partner(wb);
+                e_part += pair_term2(xo, xo, xa, xb, pa, pb, (wa >> 24) & 1, (wb >> 24) & 1, fa, fb);
+            }
+            if (r < lig.n_rounds) {
+                const uint32_t w = __ldg(rw + 32 * r);
+                const float3 xj = partner(w);
+                e_part += pair_term(make_float4(xo.x, xo.y, xo.z, 0.f),
+                                    make_float4(xj.x, xj.y, xj.z, 0.f), __ldg(rc + 32 * r),
+                                    (w >> 24) & 1, fa);
+            }
+        } else {
+            group_sync<TPP>(group);
+            int p = gt;
+            float3 fa, fb;
+            for (; p + TPP < NP; p += 2 * TPP) {  // pairs p and p + TPP, packed arithmetic
+                const uint32_t pa = prs[p], pb = prs[p + TPP];
+                e_part += pair_term2(xyz3(xyz[pa & 255]), xyz3(xyz[pb & 255]),
+                                     xyz3(xyz[(pa >> 8) & 255]), xyz3(xyz[(pb >> 8) & 255]),
+                                     __ldg(pconst + p), __ldg(pconst + p + TPP), (pa >> 24) & 1,
+                                     (pb >> 24) & 1, fa, fb);
+            }
+            if (p < NP) {
+                const uint32_t pr = prs[p];
+                e_part += pair_term(xyz[pr & 255], xyz[(pr >> 8) & 255], __ldg(pconst + p),
+                                    (pr >> 24) & 1, fa);
+            }
         }
-        if (p < NP) {
-            const uint32_t pr = prs[p];
-            float3 f;
-            e_part += pair_term(xyz[pr & 255], xyz[(pr >> 8) & 255], __ldg(pconst + p),
-                                (pr >> 24) & 1, f);
+        if constexpr (VAR == ADGB_REDUCE_SHFL) {   // one value: a butterfly
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) e_part += __shfl_xor_sync(0xffffffffu, e_part, off);
+            if constexpr (TPP > 32) {
+                if ((gt & 31) == 0) red[gt >> 5] = e_part;
+                group_sync<TPP>(group);
+                e_part = red[0];
+#pragma unroll
+                for (int w = 1; w < TPP / 32; w++) e_part += red[w];
+            }
+        } else {
+            float v[8] = {e_part, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            group_sum8<TPP, VAR>(v, red, stage, group, gt, tw);
+            e_part = v[0];
         }
-        float v[8] = {e_part, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        group_sum8<TPP, VAR>(v, red, stage, group, gt, tw);
-        group_sync<TPP>(group);   // every lane is done with genes_s, sc and xyz
-        return v[0];
+        group_sync<TPP>(group);   // every lane is done with genes_s, sc, xyz and red
+        return e_part;
     };
 
     float *gio = a.genes + (size_t)pose * G;
