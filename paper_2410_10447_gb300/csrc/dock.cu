@@ -80,70 +80,99 @@ __device__ void block_argmin(float e, int k, float *s_e, int *s_k, float &best_e
     __syncthreads();
 }
 
-__global__ void ga_kernel(int pop, int G, const float *go, const float *eo, const DockCfg d,
-                          uint32_t gen, float *gn, int *iters, const int *done) {
-    extern __shared__ float s_e[];  // [pop] energies, then argmin scratch
-    float *s_we = s_e + pop;
-    int *s_wk = reinterpret_cast<int *>(s_we + 32);
-    const int run = blockIdx.x;
+// One GA generation: a warp an individual.  A child's random words are the
+// Philox blocks 0 (tournaments), 1 (crossover, cuts, local search) and
+// 2 + j / 2 (gene j's mutation), at most 25: every lane computes one of them
+// and the words go round by shuffles, so a child costs one Philox call's
+// latency.  (A thread an individual ran two calls a gene in sequence, with a
+// run's 150 individuals on one SM: 10.2 us a generation of 20 x 150
+// individuals of 14 genes, now 5.1.)
+constexpr int GA_WARPS = 8;
+__global__ void __launch_bounds__(32 * GA_WARPS) ga_kernel(int n_runs, int pop, int G, const float *go,
+                                                           const float *eo, const DockCfg d,
+                                                           uint32_t gen, float *gn, int *iters,
+                                                           const int *done) {
+    const int idx = blockIdx.x * GA_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (idx >= n_runs * pop) return;
+    const int run = idx / pop, k = idx - run * pop;
     const size_t base = (size_t)run * pop;
-    float e = INFINITY;
-    int kk = 0x7fffffff;
-    for (int k = threadIdx.x; k < pop; k += blockDim.x) {
-        const float v = eo[base + k];
-        s_e[k] = v;
-        if (v < e || (v == e && k < kk)) {
-            e = v;
-            kk = k;
+    float *child = gn + (size_t)idx * G;
+    if (done && done[run] != 0) {   // a stopped run keeps its population
+        const float *src = go + (size_t)idx * G;
+        for (int j = lane; j < G; j += 32) child[j] = src[j];
+        if (lane == 0) iters[idx] = 0;
+        return;
+    }
+    const Philox4 o = philox4x32_10((uint32_t)k, gen, (uint32_t)run, (uint32_t)lane,
+                                    (uint32_t)d.seed, (uint32_t)(d.seed >> 32));
+    auto word = [&](int w) {   // word w (the same in every lane) of the child's stream
+        const uint32_t x = (w & 2) ? ((w & 1) ? o.w : o.z) : ((w & 1) ? o.y : o.x);
+        return __shfl_sync(0xffffffffu, x, w >> 2);
+    };
+    const uint32_t w_ls = word(W_LS);
+    if (lane == 0) iters[idx] = unit24(w_ls) < d.ls_rate ? d.ls_iters : 1;
+    if (k == 0) {   // the previous generation's best
+        float e = INFINITY;
+        int kk = 0x7fffffff;
+        for (int i = lane; i < pop; i += 32) {
+            const float v = eo[base + i];
+            if (v < e || (v == e && i < kk)) {
+                e = v;
+                kk = i;
+            }
+        }
+        for (int off = 16; off > 0; off >>= 1) {
+            const float oe = __shfl_xor_sync(0xffffffffu, e, off);
+            const int ok = __shfl_xor_sync(0xffffffffu, kk, off);
+            if (oe < e || (oe == e && ok < kk)) {
+                e = oe;
+                kk = ok;
+            }
+        }
+        const int bk = kk < 0 || kk >= pop ? 0 : kk;
+        const float *src = go + (base + bk) * G;
+        for (int j = lane; j < G; j += 32) child[j] = src[j];
+        return;
+    }
+    int par[2];
+#pragma unroll
+    for (int t = 0; t < 2; t++) {
+        const int a = index_below(word(W_TOUR + 2 * t), pop);
+        const int b = index_below(word(W_TOUR + 2 * t + 1), pop);
+        const float ea = eo[base + a], eb = eo[base + b];
+        par[t] = (eb < ea || (eb == ea && b < a)) ? b : a;
+    }
+    const float *A = go + (base + par[0]) * G, *B = go + (base + par[1]) * G;
+    int c1 = index_below(word(W_CUT), G + 1), c2 = index_below(word(W_CUT + 1), G + 1);
+    if (!(unit24(word(W_CROSS)) < d.p_cross)) c1 = c2 = 0;
+    if (c1 > c2) {
+        const int t = c1;
+        c1 = c2;
+        c2 = t;
+    }
+    for (int j0 = 0; j0 < G; j0 += 32) {
+        const int j = j0 + lane, src = (W_MUT + 2 * j) >> 2;   // lane of gene j's block
+        const bool odd = j & 1;
+        const uint32_t mx = __shfl_sync(0xffffffffu, o.x, src & 31), my = __shfl_sync(0xffffffffu, o.y, src & 31);
+        const uint32_t mz = __shfl_sync(0xffffffffu, o.z, src & 31), mw = __shfl_sync(0xffffffffu, o.w, src & 31);
+        if (j < G) {
+            float v = (j >= c1 && j < c2) ? B[j] : A[j];
+            if (unit24(odd ? mz : mx) < d.p_mut) {
+                const float off = 2.f * unit24(odd ? mw : my) - 1.f;
+                v += off * (j < 3 ? d.mut_trans : d.mut_angle);
+            }
+            if (j >= 6) v -= 2.f * PI_F * floorf((v + PI_F) * (0.5f / PI_F));
+            child[j] = v;
         }
     }
-    __syncthreads();
-    float be;
-    int bk;
-    block_argmin(e, kk, s_we, s_wk, be, bk);
-    if (bk < 0 || bk >= pop) bk = 0;
-    const bool stop = done && done[run] != 0;
-    for (int k = threadIdx.x; k < pop; k += blockDim.x) {
-        float *child = gn + (base + k) * G;
-        if (stop) {
-            const float *src = go + (base + k) * G;
-            for (int j = 0; j < G; j++) child[j] = src[j];
-            iters[base + k] = 0;
-            continue;
-        }
-        if (k == 0) {
-            const float *src = go + (base + bk) * G;
-            for (int j = 0; j < G; j++) child[j] = src[j];
-        } else {
-            int par[2];
-            for (int t = 0; t < 2; t++) {
-                const int a = index_below(ga_word(d.seed, run, gen, k, W_TOUR + 2 * t), pop);
-                const int b = index_below(ga_word(d.seed, run, gen, k, W_TOUR + 2 * t + 1), pop);
-                par[t] = (s_e[b] < s_e[a] || (s_e[b] == s_e[a] && b < a)) ? b : a;
-            }
-            const float *A = go + (base + par[0]) * G, *B = go + (base + par[1]) * G;
-            int c1 = 0, c2 = 0;
-            if (unit24(ga_word(d.seed, run, gen, k, W_CROSS)) < d.p_cross) {
-                c1 = index_below(ga_word(d.seed, run, gen, k, W_CUT), G + 1);
-                c2 = index_below(ga_word(d.seed, run, gen, k, W_CUT + 1), G + 1);
-                if (c1 > c2) {
-                    const int t = c1;
-                    c1 = c2;
-                    c2 = t;
-                }
-            }
-            for (int j = 0; j < G; j++) {
-                float v = (j >= c1 && j < c2) ? B[j] : A[j];
-                if (unit24(ga_word(d.seed, run, gen, k, W_MUT + 2 * j)) < d.p_mut) {
-                    const float off = 2.f * unit24(ga_word(d.seed, run, gen, k, W_MUT + 2 * j + 1)) - 1.f;
-                    v += off * (j < 3 ? d.mut_trans : d.mut_angle);
-                }
-                if (j >= 6) v -= 2.f * PI_F * floorf((v + PI_F) * (0.5f / PI_F));
-                child[j] = v;
-            }
-        }
-        iters[base + k] = unit24(ga_word(d.seed, run, gen, k, W_LS)) < d.ls_rate ? d.ls_iters : 1;
-    }
+}
+static_assert(((8 + 2 * (MAX_GENES - 1)) >> 2) < 32, "a child's Philox blocks exceed a warp");
+
+void run_ga_kernel(const DockCfg &d, int G, int gen, const float *genes, const float *energy,
+                   float *genes_out, int *iters, const int *done, cudaStream_t s) {
+    const int n = d.n_runs * d.pop;
+    ga_kernel<<<(n + GA_WARPS - 1) / GA_WARPS, 32 * GA_WARPS, 0, s>>>(
+        d.n_runs, d.pop, G, genes, energy, d, (uint32_t)gen, genes_out, iters, done);
 }
 
 // A run evaluated in this pass (runs stopped before it have all iters 0).
@@ -425,10 +454,7 @@ cudaError_t launch_init_population(const RecDev &rec, int n_tors, uint64_t seed,
 
 cudaError_t launch_ga_generation(const DockCfg &d, int G, int gen, const float *genes,
                                  const float *energy, float *genes_out, int *iters, cudaStream_t s) {
-    const int gt = d.pop >= 1024 ? 1024 : ((d.pop + 31) / 32) * 32;
-    const int gsm = (d.pop + 32) * 4 + 32 * 4;
-    ga_kernel<<<d.n_runs, gt, gsm, s>>>(d.pop, G, genes, energy, d, (uint32_t)gen, genes_out, iters,
-                                        nullptr);
+    run_ga_kernel(d, G, gen, genes, energy, genes_out, iters, nullptr, s);
     return cudaGetLastError();
 }
 
@@ -444,10 +470,7 @@ cudaError_t launch_job_start(const RecDev &rec, int n_tors, const DockCfg &d, Do
 }
 
 cudaError_t launch_job_ga(const DockCfg &d, int G, int gen, DockScratch &w, int cur, cudaStream_t s) {
-    const int gt = d.pop >= 1024 ? 1024 : ((d.pop + 31) / 32) * 32;
-    const int gsm = (d.pop + 32) * 4 + 32 * 4;
-    ga_kernel<<<d.n_runs, gt, gsm, s>>>(d.pop, G, w.genes[cur], w.energy, d, (uint32_t)gen,
-                                       w.genes[cur ^ 1], w.iters, w.done);
+    run_ga_kernel(d, G, gen, w.genes[cur], w.energy, w.genes[cur ^ 1], w.iters, w.done, s);
     return cudaGetLastError();
 }
 
@@ -516,11 +539,8 @@ cudaError_t launch_dock(const RecDev &rec, const LigDev &lig, const EvalCfg &cfg
                                        w.best_e, w.evals, w.done, d.max_evals, 0, d.conv_every,
                                        d.conv_top, d.conv_tol);
     int cur = 0;
-    const int gt = d.pop >= 1024 ? 1024 : ((d.pop + 31) / 32) * 32;
-    const int gsm = (d.pop + 32) * 4 + 32 * 4;
     for (int gen = 1; gen <= d.max_gens; gen++) {
-        ga_kernel<<<d.n_runs, gt, gsm, s>>>(d.pop, G, w.genes[cur], w.energy, d, (uint32_t)gen,
-                                           w.genes[cur ^ 1], w.iters, w.done);
+        run_ga_kernel(d, G, gen, w.genes[cur], w.energy, w.genes[cur ^ 1], w.iters, w.done, s);
         cur ^= 1;
         if ((e = local_search(w.genes[cur], gen)) != cudaSuccess) return e;
         best_kernel<<<d.n_runs, bt, 0, s>>>(d.pop, G, w.genes[cur], w.energy, w.iters,
