@@ -326,53 +326,65 @@ __device__ __forceinline__ void drot(D3 &r, D3 c, D3 k, double s, double omc) {
 }
 
 // Energy of one genotype in double precision (coordinates, grid terms and
-// pair terms recomputed from the stored single-precision inputs).  One warp
-// per genotype; coordinates in shared memory.
-__global__ void rescore_fp64_kernel(const RecDev R, const LigDev L, int n, const float *genes,
-                                    double *out) {
-    extern __shared__ double s_x[];  // [warps][N][3]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int pose = blockIdx.x * (blockDim.x >> 5) + warp;
-    if (pose >= n) return;
+// pair terms recomputed from the stored single-precision inputs).  A block a
+// genotype: double precision runs at 1/64 of the single rate here, so a
+// genotype's chain of sines, divisions and exponentials is what takes the
+// time.  Each torsion's axis and sine are computed once (not once an atom and
+// torsion) and the pairs spread over 256 threads: 20 genotypes of 32 atoms 88
+// us with a warp each, now 38; of 256 atoms 4742 -> 1086.
+constexpr int RESCORE_THREADS = 256;
+__global__ void __launch_bounds__(RESCORE_THREADS) rescore_fp64_kernel(const RecDev R, const LigDev L,
+                                                                       const float *genes, double *out) {
+    __shared__ double X[3 * ADGB_MAX_ATOMS];
+    __shared__ D3 s_ax[ADGB_MAX_TORS + 1];                             // unit axes; [T]: the rigid one
+    __shared__ double s_s[ADGB_MAX_TORS + 1], s_o[ADGB_MAX_TORS + 1];  // sin, 1 - cos
+    __shared__ double s_e[RESCORE_THREADS / 32];
+    const int pose = blockIdx.x, t = threadIdx.x;
     const int N = L.n_atoms, T = L.n_tors, G = 6 + T;
-    double *X = s_x + (size_t)warp * N * 3;
     const float *g = genes + (size_t)pose * G;
-    const double phi = g[3], th = g[4], al = g[5];
-    const D3 u = {sin(th) * cos(phi), sin(th) * sin(phi), cos(th)};
-    const double sa = sin(al), oca = 1.0 - cos(al);
-    for (int i = lane; i < N; i += 32) {
+    // torsions one a lane over all warps; the rigid rotation on the last warp
+    if (t < T) {
+        const int4 ta = L.tatoms[t];
+        const float4 a4 = L.ref[ta.x], b4 = L.ref[ta.y];
+        D3 ax = {(double)b4.x - a4.x, (double)b4.y - a4.y, (double)b4.z - a4.z};
+        const double l = sqrt(ax.x * ax.x + ax.y * ax.y + ax.z * ax.z);
+        ax.x /= l;
+        ax.y /= l;
+        ax.z /= l;
+        s_ax[t] = ax;
+        const double psi = g[6 + t];
+        s_s[t] = sin(psi);
+        s_o[t] = 1.0 - cos(psi);
+    }
+    if (t == RESCORE_THREADS - 32) {
+        const double phi = g[3], th = g[4], al = g[5];
+        s_ax[T] = {sin(th) * cos(phi), sin(th) * sin(phi), cos(th)};
+        s_s[T] = sin(al);
+        s_o[T] = 1.0 - cos(al);
+    }
+    __syncthreads();
+    double e = 0.0;
+    const int nn[3] = {R.nx, R.ny, R.nz};
+    for (int i = t; i < N; i += RESCORE_THREADS) {
         const float4 r4 = L.ref[i];
         D3 p = {r4.x, r4.y, r4.z};
         for (int k = L.frag[i]; k >= 0; k = L.tparent[k]) {
-            const int4 ta = L.tatoms[k];
-            const float4 a4 = L.ref[ta.x], b4 = L.ref[ta.y];
-            D3 ax = {(double)b4.x - a4.x, (double)b4.y - a4.y, (double)b4.z - a4.z};
-            const double l = sqrt(ax.x * ax.x + ax.y * ax.y + ax.z * ax.z);
-            ax.x /= l;
-            ax.y /= l;
-            ax.z /= l;
-            const double psi = g[6 + k];
-            drot(p, D3{b4.x, b4.y, b4.z}, ax, sin(psi), 1.0 - cos(psi));
+            const float4 b4 = L.ref[L.tatoms[k].y];
+            drot(p, D3{b4.x, b4.y, b4.z}, s_ax[k], s_s[k], s_o[k]);
         }
-        drot(p, D3{0.0, 0.0, 0.0}, u, sa, oca);
-        X[3 * i] = p.x + g[0];
-        X[3 * i + 1] = p.y + g[1];
-        X[3 * i + 2] = p.z + g[2];
-    }
-    __syncwarp();
-    double e = 0.0;
-    const int nn[3] = {R.nx, R.ny, R.nz};
-    for (int i = lane; i < N; i += 32) {
-        const double q = L.ref[i].w, aq = fabs(q);
-        const int t = L.type[i];
-        double pc[3], f[3], pen = 0.0;
+        drot(p, D3{0.0, 0.0, 0.0}, s_ax[T], s_s[T], s_o[T]);
+        const double xs[3] = {p.x + g[0], p.y + g[1], p.z + g[2]};
+        const double q = r4.w, aq = fabs(q);
+        const int type = L.type[i];
+        double f[3], pen = 0.0;
         int i0[3];
         for (int d = 0; d < 3; d++) {
-            const double xv = X[3 * i + d];
+            const double xv = xs[d];
+            X[3 * i + d] = xv;
             const double lo = R.lo[d], hi = (double)R.lo[d] + (double)(nn[d] - 1) * (double)R.h;
-            pc[d] = xv < lo ? lo : (xv > hi ? hi : xv);
-            pen += (xv - pc[d]) * (xv - pc[d]);
-            const double uu = (pc[d] - lo) / (double)R.h;
+            const double pc = xv < lo ? lo : (xv > hi ? hi : xv);
+            pen += (xv - pc) * (xv - pc);
+            const double uu = (pc - lo) / (double)R.h;
             int c = (int)floor(uu);
             c = c < 0 ? 0 : (c > nn[d] - 2 ? nn[d] - 2 : c);
             i0[d] = c;
@@ -384,12 +396,13 @@ __global__ void rescore_fp64_kernel(const RecDev R, const LigDev L, int n, const
         for (int c = 0; c < 8; c++) {
             const int cx = c & 1, cy = (c >> 1) & 1, cz = c >> 2;
             const double w = (cx ? f[0] : 1.0 - f[0]) * (cy ? f[1] : 1.0 - f[1]) * (cz ? f[2] : 1.0 - f[2]);
-            v += w * ((double)cp[8 * t + c] + q * (double)cp[8 * (R.M - 2) + c] +
+            v += w * ((double)cp[8 * type + c] + q * (double)cp[8 * (R.M - 2) + c] +
                       aq * (double)cp[8 * (R.M - 1) + c]);
         }
         e += v + D_W_OUT * pen;
     }
-    for (int p = lane; p < L.n_pairs; p += 32) {
+    __syncthreads();
+    for (int p = t; p < L.n_pairs; p += RESCORE_THREADS) {
         const uint32_t pr = L.pairs[p];
         const int i = pr & 255, j = (pr >> 8) & 255;
         const int ti = L.type[i], tj = L.type[j];
@@ -420,7 +433,12 @@ __global__ void rescore_fp64_kernel(const RecDev R, const LigDev L, int n, const
         e += ev + eel + eds;
     }
     for (int off = 16; off > 0; off >>= 1) e += __shfl_xor_sync(0xffffffffu, e, off);
-    if (lane == 0) out[pose] = e;
+    if ((t & 31) == 0) s_e[t >> 5] = e;
+    __syncthreads();
+    if (t == 0) {
+        for (int w = 1; w < RESCORE_THREADS / 32; w++) e += s_e[w];
+        out[pose] = e;
+    }
 }
 
 // Raw Philox4x32-10 words: in [n][6] = (counter 0-3, key 0-1), out [n][4].
@@ -491,9 +509,7 @@ cudaError_t launch_ga_converged(int n_runs, int pop, int top, float tol, const f
 cudaError_t launch_rescore_fp64(const RecDev &rec, const LigDev &lig, int n, const float *genes,
                                 double *out, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    const int warps = 4;
-    const int smem = warps * lig.n_atoms * 3 * (int)sizeof(double);
-    rescore_fp64_kernel<<<(n + warps - 1) / warps, 32 * warps, smem, s>>>(rec, lig, n, genes, out);
+    rescore_fp64_kernel<<<n, RESCORE_THREADS, 0, s>>>(rec, lig, genes, out);
     return cudaGetLastError();
 }
 
