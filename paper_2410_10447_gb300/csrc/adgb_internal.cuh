@@ -379,6 +379,36 @@ inline void prefer_l1(int smem, int threads) {
     else (void)cudaGetLastError();
 }
 
+// Programmatic dependent launches: a kernel launched by launch_dependent may
+// start while the kernel before it on the stream still runs (once each of that
+// one's blocks has called dependents_may_start), and calls
+// wait_for_predecessor before it touches anything but a ligand's or receptor's
+// uploaded, unchanging tables.  So the launch and the copy of the ligand's
+// constants into shared memory overlap with the end of the kernel before.
+// Not for the tcgen05 forms: a waiting block would hold tensor memory that a
+// block of the kernel it waits for may still need.
+__device__ __forceinline__ void dependents_may_start() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+__device__ __forceinline__ void wait_for_predecessor() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_dependent(void (*k)(P...), int grid, int block, int smem, cudaStream_t s,
+                                    A... args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Dynamic shared memory a launch may take without asking for more.
 constexpr int SMEM_DEFAULT_LIMIT = 46 * 1024;   // of 48 KB, static shared memory included
 template <typename K>

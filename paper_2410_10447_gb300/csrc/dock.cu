@@ -92,6 +92,8 @@ __global__ void __launch_bounds__(32 * GA_WARPS) ga_kernel(int n_runs, int pop, 
                                                            const float *eo, const DockCfg d,
                                                            uint32_t gen, float *gn, int *iters,
                                                            const int *done) {
+    dependents_may_start();
+    wait_for_predecessor();
     const int idx = blockIdx.x * GA_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (idx >= n_runs * pop) return;
     const int run = idx / pop, k = idx - run * pop;
@@ -168,11 +170,11 @@ __global__ void __launch_bounds__(32 * GA_WARPS) ga_kernel(int n_runs, int pop, 
 }
 static_assert(((8 + 2 * (MAX_GENES - 1)) >> 2) < 32, "a child's Philox blocks exceed a warp");
 
-void run_ga_kernel(const DockCfg &d, int G, int gen, const float *genes, const float *energy,
+cudaError_t run_ga_kernel(const DockCfg &d, int G, int gen, const float *genes, const float *energy,
                    float *genes_out, int *iters, const int *done, cudaStream_t s) {
     const int n = d.n_runs * d.pop;
-    ga_kernel<<<(n + GA_WARPS - 1) / GA_WARPS, 32 * GA_WARPS, 0, s>>>(
-        d.n_runs, d.pop, G, genes, energy, d, (uint32_t)gen, genes_out, iters, done);
+    return launch_dependent(ga_kernel, (n + GA_WARPS - 1) / GA_WARPS, 32 * GA_WARPS, 0, s, d.n_runs,
+                            d.pop, G, genes, energy, d, (uint32_t)gen, genes_out, iters, done);
 }
 
 // A run evaluated in this pass (runs stopped before it have all iters 0).
@@ -251,6 +253,8 @@ __global__ void best_kernel(int pop, int G, const float *genes, const float *ene
     __shared__ long long s_n[32];
     __shared__ float s_e[1024];
     __shared__ double s_d[32];
+    dependents_may_start();
+    wait_for_predecessor();
     const int run = blockIdx.x;
     const size_t base = (size_t)run * pop;
     float e = INFINITY;
@@ -472,8 +476,7 @@ cudaError_t launch_init_population(const RecDev &rec, int n_tors, uint64_t seed,
 
 cudaError_t launch_ga_generation(const DockCfg &d, int G, int gen, const float *genes,
                                  const float *energy, float *genes_out, int *iters, cudaStream_t s) {
-    run_ga_kernel(d, G, gen, genes, energy, genes_out, iters, nullptr, s);
-    return cudaGetLastError();
+    return run_ga_kernel(d, G, gen, genes, energy, genes_out, iters, nullptr, s);
 }
 
 // The steps of dock() one at a time, for the serving loop, which advances
@@ -488,16 +491,14 @@ cudaError_t launch_job_start(const RecDev &rec, int n_tors, const DockCfg &d, Do
 }
 
 cudaError_t launch_job_ga(const DockCfg &d, int G, int gen, DockScratch &w, int cur, cudaStream_t s) {
-    run_ga_kernel(d, G, gen, w.genes[cur], w.energy, w.genes[cur ^ 1], w.iters, w.done, s);
-    return cudaGetLastError();
+    return run_ga_kernel(d, G, gen, w.genes[cur], w.energy, w.genes[cur ^ 1], w.iters, w.done, s);
 }
 
 cudaError_t launch_job_best(const DockCfg &d, int G, int gen, DockScratch &w, int cur,
                             float *best_genes, cudaStream_t s) {
-    best_kernel<<<d.n_runs, 128, 0, s>>>(d.pop, G, w.genes[cur], w.energy, w.iters, best_genes,
-                                         w.best_e, w.evals, w.done, d.max_evals, gen, d.conv_every,
-                                         d.conv_top, d.conv_tol);
-    return cudaGetLastError();
+    return launch_dependent(best_kernel, d.n_runs, 128, 0, s, d.pop, G, w.genes[cur], w.energy, w.iters,
+                            best_genes, w.best_e, w.evals, w.done, d.max_evals, gen, d.conv_every,
+                            d.conv_top, d.conv_tol);
 }
 
 cudaError_t launch_ga_converged(int n_runs, int pop, int top, float tol, const float *energy,
@@ -550,18 +551,15 @@ cudaError_t launch_dock(const RecDev &rec, const LigDev &lig, const EvalCfg &cfg
         return launch_dock_ls(rec, lig, cfg, d, genes, gen, w, s);
     };
     if ((e = local_search(w.genes[0], 0)) != cudaSuccess) return e;
-    const int bt = 128;
-    best_kernel<<<d.n_runs, bt, 0, s>>>(d.pop, G, w.genes[0], w.energy, w.iters, best_genes,
-                                       w.best_e, w.evals, w.done, d.max_evals, 0, d.conv_every,
-                                       d.conv_top, d.conv_tol);
+    if ((e = launch_job_best(d, G, 0, w, 0, best_genes, s)) != cudaSuccess) return e;
     int cur = 0;
     for (int gen = 1; gen <= d.max_gens; gen++) {
-        run_ga_kernel(d, G, gen, w.genes[cur], w.energy, w.genes[cur ^ 1], w.iters, w.done, s);
+        if ((e = run_ga_kernel(d, G, gen, w.genes[cur], w.energy, w.genes[cur ^ 1], w.iters, w.done, s)) !=
+            cudaSuccess)
+            return e;
         cur ^= 1;
         if ((e = local_search(w.genes[cur], gen)) != cudaSuccess) return e;
-        best_kernel<<<d.n_runs, bt, 0, s>>>(d.pop, G, w.genes[cur], w.energy, w.iters,
-                                           best_genes, w.best_e, w.evals, w.done, d.max_evals,
-                                           gen, d.conv_every, d.conv_top, d.conv_tol);
+        if ((e = launch_job_best(d, G, gen, w, cur, best_genes, s)) != cudaSuccess) return e;
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if ((e = launch_rescore_fp64(rec, lig, d.n_runs, best_genes, best_energy, s)) != cudaSuccess)

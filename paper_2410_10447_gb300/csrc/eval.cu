@@ -947,9 +947,11 @@ template <int TPP, int VAR>
 __global__ void __launch_bounds__(128, ADGB_MIN_BLOCKS) sw_kernel(const SwArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sm = smem_raw + tc_front<VAR>();
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
     const StagedLig sl = stage_ligand(sm, a.L, a.lig);
     Tc05Warp tw;
     tc_begin<VAR>(smem_raw, tw);
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) wait_for_predecessor();
     __syncthreads();
     const int group = threadIdx.x / TPP, gt = threadIdx.x % TPP;
     const int pose = blockIdx.x * (blockDim.x / TPP) + group;
@@ -1248,7 +1250,9 @@ static cudaError_t launch_sw_t(const SwArgs &a, int ppb, int smem, cudaStream_t 
     auto k = sw_kernel<TPP, VAR>;
     const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
-    k<<<(a.n + ppb - 1) / ppb, TPP * ppb, smem, s>>>(a);
+    const int grid = (a.n + ppb - 1) / ppb;
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) return launch_dependent(k, grid, TPP * ppb, smem, s, a);
+    k<<<grid, TPP * ppb, smem, s>>>(a);
     return cudaGetLastError();
 }
 

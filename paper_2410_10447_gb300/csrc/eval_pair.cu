@@ -831,6 +831,7 @@ __global__ void __launch_bounds__(64, 5) eval_pair_kernel(const PairArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;
     unsigned char *sm = smem_raw + (VAR == ADGB_REDUCE_TCGEN05 ? tc2_region(W) : 0);
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
     stage_pair_ligand(sm, a.L, a.lig);
     Tc2 tw;
     if constexpr (VAR == ADGB_REDUCE_TCGEN05) {
@@ -838,6 +839,7 @@ __global__ void __launch_bounds__(64, 5) eval_pair_kernel(const PairArgs a) {
         tc2_begin(smem_raw, tw);
         if constexpr ((SKIP & SK_BLOCKMMA) != 0) tw.mbar -= warp;   // warp 0's barrier for all
     }
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) wait_for_predecessor();
     __syncthreads();
     const int b0 = blockIdx.x * a.ppb;
     const int count = min(a.ppb, a.n - b0);
@@ -1041,7 +1043,9 @@ static cudaError_t launch_pair_t(const PairArgs &a, int smem, cudaStream_t s) {
     const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     if constexpr (VAR != ADGB_REDUCE_TCGEN05) prefer_l1<eval_pair_kernel<VAR, SKIP>>(smem, 32 * warps);
-    k<<<(a.n + a.ppb - 1) / a.ppb, 32 * warps, smem, s>>>(a);
+    const int grid = (a.n + a.ppb - 1) / a.ppb;
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) return launch_dependent(k, grid, 32 * warps, smem, s, a);
+    k<<<grid, 32 * warps, smem, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -562,9 +562,11 @@ template <int A, int VAR, int MB>
 __global__ void __launch_bounds__(128, MB) eval_ring_kernel(const RingArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sm = smem_raw + tc_front<VAR>();
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
     stage_ring_ligand(sm, a.L, a.lig);
     Tc05Warp tw;
     tc_begin<VAR>(smem_raw, tw);
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) wait_for_predecessor();
     __syncthreads();
     const int G = 6 + a.lig.n_tors, p0 = 2 * blockIdx.x;
     PairIO io;
@@ -630,6 +632,8 @@ cudaError_t launch_ring_t(const RingArgs &a, int threads, int smem, cudaStream_t
     auto k = eval_ring_kernel<A, VAR, MB>;
     const cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05)
+        return launch_dependent(k, (a.n + 1) / 2, threads, smem, s, a);
     k<<<(a.n + 1) / 2, threads, smem, s>>>(a);
     return cudaGetLastError();
 }
