@@ -551,13 +551,17 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
     }
 }
 
-// Resident blocks of 128 threads an SM the kernels are built for (MB): 4, at
-// 128 registers a thread, or 5 at 96, which spill a little outside the sweep.
-// 5 for a = 3 up to 96 atoms where the launch fills more than 4 blocks an SM
-// (12 000 genotypes of 45 atoms 176 -> 186M evaluations/s, of 90 atoms 84.0 ->
-// 86.4M; 1500 of 90 atoms, one wave instead of two, 67 -> 80M); where 4 blocks
-// an SM hold the launch they run 3% faster (45 atoms x 1000), and above 160
-// atoms shared memory allows no fifth (256 atoms 13.7 -> 12.2M).
+// Resident blocks of 128 threads an SM the kernels are built for (MB), i.e.
+// registers a thread: 2 (254), 3 (168), 4 (128) or, for a = 3, 5 (96, a little
+// spilled outside the sweep).  All give the same bits.  A launch that needs no
+// more blocks an SM takes the kernel with more registers, whose loads and pair
+// chains overlap better (M evaluations/s, shuffle form, 4 -> 3 -> 2 blocks;
+// 300 genotypes, one block an SM: 45 atoms 60 -> 64 -> 64, 90 33 -> 37 -> 39,
+// 160 14 -> 16 -> 21, 256 - -> 7.9 -> 10.0; 900 genotypes, three: 45 atoms 148
+// -> 155, 160 30 -> 33).  Larger launches: 5 for a = 3 up to 96 atoms (12 000
+// genotypes of 45 atoms 176 -> 186, of 90 atoms 84.0 -> 86.4), 3 from 250
+// atoms on (256 x 8192 15.4 -> 16.8: a fourth block's shared memory leaves the
+// L1 cache 20 KB), else 4.
 template <int A, int VAR, int MB>
 __global__ void __launch_bounds__(128, MB) eval_ring_kernel(const RingArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -638,16 +642,30 @@ cudaError_t launch_ring_t(const RingArgs &a, int threads, int smem, cudaStream_t
     return cudaGetLastError();
 }
 
-template <int A, int MB>
-cudaError_t launch_ring_v(const RingArgs &a, int variant, int threads, int smem, cudaStream_t s) {
+// need: blocks an SM that hold the whole launch at once.
+template <int A, int VAR>
+cudaError_t launch_ring_mb(const RingArgs &a, int need, int threads, int smem, cudaStream_t s) {
+    if constexpr (VAR == ADGB_REDUCE_SHFL) {
+        if (need <= 2) return launch_ring_t<A, VAR, 2>(a, threads, smem, s);
+        if (need <= 3 || (need > 4 && a.lig.n_atoms >= 250))
+            return launch_ring_t<A, VAR, 3>(a, threads, smem, s);
+    }
+    if constexpr (A == 3)
+        if (need > 4 && a.lig.n_atoms <= 96) return launch_ring_t<A, VAR, 5>(a, threads, smem, s);
+    return launch_ring_t<A, VAR, 4>(a, threads, smem, s);
+}
+
+template <int A>
+cudaError_t launch_ring_v(const RingArgs &a, int variant, int need, int threads, int smem,
+                          cudaStream_t s) {
     switch (variant) {
-        case ADGB_REDUCE_SHFL: return launch_ring_t<A, ADGB_REDUCE_SHFL, MB>(a, threads, smem, s);
+        case ADGB_REDUCE_SHFL: return launch_ring_mb<A, ADGB_REDUCE_SHFL>(a, need, threads, smem, s);
         case ADGB_REDUCE_MMA_TF32X2:
-            return launch_ring_t<A, ADGB_REDUCE_MMA_TF32X2, MB>(a, threads, smem, s);
+            return launch_ring_mb<A, ADGB_REDUCE_MMA_TF32X2>(a, need, threads, smem, s);
         case ADGB_REDUCE_MMA_BF16X3:
-            return launch_ring_t<A, ADGB_REDUCE_MMA_BF16X3, MB>(a, threads, smem, s);
+            return launch_ring_mb<A, ADGB_REDUCE_MMA_BF16X3>(a, need, threads, smem, s);
         case ADGB_REDUCE_TCGEN05:
-            return launch_ring_t<A, ADGB_REDUCE_TCGEN05, MB>(a, threads, smem, s);
+            return launch_ring_mb<A, ADGB_REDUCE_TCGEN05>(a, need, threads, smem, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -728,14 +746,13 @@ cudaError_t launch_eval_ring(const RecDev &rec, const LigDev &lig, const EvalCfg
     if (e != cudaSuccess) return e;
     const int smem = tc_smem_bytes(a.L.total, rs.warps, cfg.variant, dev);
     if (smem < 0) return cudaErrorInvalidValue;
-    if (rs.a == 5) return launch_ring_v<5, 4>(a, cfg.variant, 32 * rs.warps, smem, s);
-    if (rs.a == 4) return launch_ring_v<4, 4>(a, cfg.variant, 32 * rs.warps, smem, s);
     int sms = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    if (lig.n_atoms <= 96 && (n + 1) / 2 > 4 * sms)
-        return launch_ring_v<3, 5>(a, cfg.variant, 32 * rs.warps, smem, s);
-    return launch_ring_v<3, 4>(a, cfg.variant, 32 * rs.warps, smem, s);
+    const int need = ((n + 1) / 2 + sms - 1) / sms;
+    if (rs.a == 3) return launch_ring_v<3>(a, cfg.variant, need, 32 * rs.warps, smem, s);
+    if (rs.a == 4) return launch_ring_v<4>(a, cfg.variant, need, 32 * rs.warps, smem, s);
+    return launch_ring_v<5>(a, cfg.variant, need, 32 * rs.warps, smem, s);
 }
 
 cudaError_t ring_tc_gave_up_async(unsigned int *dst, cudaStream_t s) {

@@ -103,6 +103,24 @@ def test_ring_genotype_does_not_depend_on_its_partner(pkg, rec):
     ctx.close()
 
 
+@pytest.mark.parametrize("n_atoms", [40, 60, 70, 256])
+def test_ring_bits_do_not_depend_on_the_launch_size(pkg, rec, n_atoms):
+    """Launches of 1 to 6 blocks an SM run kernels of different register
+    budgets: a genotype's bits are the same in each."""
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    lig = synth.make_ligand(49_000 + n_atoms, n_atoms, 4, 8)
+    first = synth.make_poses(49_001, 6, rec, 8)
+    ctx = pkg.Context(0)
+    rid, lid = ctx.upload_receptor_grids(rec), ctx.upload_ligand_torsion_tree(lig)
+    ref = ctx.local_search(rid, lid, first.copy(), 6)
+    for blocks in (2, 3, 4, 6):
+        genes = np.tile(first, (2 * sms * blocks // 6 - 1, 1))
+        b, g, _ = ctx.local_search(rid, lid, genes.copy(), 6)
+        assert np.array_equal(b[-6:], ref[0]) and np.array_equal(g[-6:], ref[1]), blocks
+    ctx.close()
+
+
 def test_ring_mixed_iteration_counts(pkg, rec):
     """LGA with half of the individuals locally searched: both genotypes of a
     block may stop at different iterations; evaluation counts as the oracle's."""
