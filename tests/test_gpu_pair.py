@@ -203,3 +203,20 @@ def test_block_mma_design_equals_warp_mma(pkg, torch, cfg1):
         ctx.ls_ablation_dev(rid, lid, g, best, 25, 3, 512)
     ctx.device_status()
     ctx.close()
+
+
+@pytest.mark.parametrize("variant", [0, 3])
+def test_bits_do_not_depend_on_the_launch_size(pkg, torch, cfg1, variant):
+    """Launches of up to 4 blocks an SM run a kernel of another register
+    budget than larger ones: a genotype's bits are the same in both."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ctx = pkg.Context(0)
+    rid = ctx.upload_receptor_grids(cfg1["receptor"])
+    lid = ctx.upload_ligand_torsion_tree(cfg1["ligand"])
+    first = cfg1["genes"][:8]
+    ref = ctx.local_search(rid, lid, first.copy(), 8, variant=variant)
+    for n in (16 * sms, 16 * sms + 8):   # 4 genotypes a block: the last small and the first large launch
+        genes = np.tile(first, (n // 8, 1))
+        b, g, _ = ctx.local_search(rid, lid, genes, 8, variant=variant)
+        assert np.array_equal(b[-8:], ref[0]) and np.array_equal(g[-8:], ref[1]), n
+    ctx.close()
