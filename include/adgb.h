@@ -403,12 +403,14 @@ int rescore_fp64_dev(adgb_ctx *ctx, int receptor_id, int ligand_id, const float 
 
 /*
  * Uneven batches: genotypes of many ligands (of different atom, torsion and
- * pair counts), each against its own receptor, locally searched by ONE
- * persistent multi-ligand launch.  Blocks take work items (up to
- * poses-per-block genotypes of one ligand, longest first) from a device
- * counter, so big and small ligands share the GPU without stragglers.  The
- * launch is captured into a CUDA graph on the first call and replayed by
- * later calls with the same buffers and parameters.
+ * pair counts), each against its own receptor, locally searched by one
+ * multi-ligand call.  Every kind of ligand the batch holds (up to 32 atoms;
+ * larger ones by the ring sweep's 3, 4 or 5 atoms a lane) is one launch over
+ * its work items (a few genotypes of one ligand, longest first), and the
+ * launches run side by side, so big and small ligands share the GPU without
+ * stragglers; a context with a launch shape of its own runs one persistent
+ * launch over all items.  The launches are captured into a CUDA graph on the
+ * first call and replayed by later calls with the same buffers and parameters.
  *
  * batch_create - item i: n_poses[i] genotypes of ligand ligand_ids[i]
  *   against receptor receptor_ids[i].  Genotypes of item i occupy rows

@@ -92,7 +92,6 @@ __global__ void __launch_bounds__(32 * GA_WARPS) ga_kernel(int n_runs, int pop, 
                                                            const float *eo, const DockCfg d,
                                                            uint32_t gen, float *gn, int *iters,
                                                            const int *done) {
-    dependents_may_start();
     wait_for_predecessor();
     const int idx = blockIdx.x * GA_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (idx >= n_runs * pop) return;

@@ -950,7 +950,6 @@ template <int TPP, int VAR, int MB>
 __global__ void __launch_bounds__(128, MB) sw_kernel(const SwArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sm = smem_raw + tc_front<VAR>();
-    if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
     const StagedLig sl = stage_ligand(sm, a.L, a.lig);
     Tc05Warp tw;
     tc_begin<VAR>(smem_raw, tw);
@@ -960,6 +959,7 @@ __global__ void __launch_bounds__(128, MB) sw_kernel(const SwArgs a) {
     const int pose = blockIdx.x * (blockDim.x / TPP) + group;
     if (pose < a.n) search_pose_sw<TPP, VAR>(sm, a.L, a.lig, a.rec, sl, group, gt, a, pose, tw);
     tc_end<VAR>(tw);
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
 }
 
 template <int TPP, int VAR, int NGS>

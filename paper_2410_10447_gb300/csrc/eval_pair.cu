@@ -836,7 +836,6 @@ __global__ void __launch_bounds__(64, MB) eval_pair_kernel(const PairArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     const int W = blockDim.x >> 5, warp = threadIdx.x >> 5;
     unsigned char *sm = smem_raw + (VAR == ADGB_REDUCE_TCGEN05 ? tc2_region(W) : 0);
-    if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
     stage_pair_ligand(sm, a.L, a.lig);
     Tc2 tw;
     if constexpr (VAR == ADGB_REDUCE_TCGEN05) {
@@ -853,6 +852,8 @@ __global__ void __launch_bounds__(64, MB) eval_pair_kernel(const PairArgs a) {
         search_pair<VAR, SKIP>(sm, a.L, a.lig, a.rec, warp, pair_io(a, p0, nvalid), tw);
     if constexpr (VAR == ADGB_REDUCE_TCGEN05)
         tc2_end<(SKIP & SK_NOISSUE) ? TC2_TEST_LIMIT : TC05_WAIT_LIMIT>(tw);
+    else
+        dependents_may_start();
 }
 
 // Persistent multi-ligand form (batches and serving): blocks take work items

@@ -566,7 +566,6 @@ template <int A, int VAR, int MB>
 __global__ void __launch_bounds__(128, MB) eval_ring_kernel(const RingArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *sm = smem_raw + tc_front<VAR>();
-    if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
     stage_ring_ligand(sm, a.L, a.lig);
     Tc05Warp tw;
     tc_begin<VAR>(smem_raw, tw);
@@ -591,6 +590,7 @@ __global__ void __launch_bounds__(128, MB) eval_ring_kernel(const RingArgs a) {
     io.eps = a.eps;
     search_ring<A, VAR>(sm, a.L, a.lig, a.rec, io, tw);
     tc_end<VAR>(tw);
+    if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
 }
 
 // Multi-ligand form (batches): block b searches work item b (up to two
