@@ -560,8 +560,11 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
 // 160 14 -> 16 -> 21, 256 - -> 7.9 -> 10.0; 900 genotypes, three: 45 atoms 148
 // -> 155, 160 30 -> 33).  Larger launches: 5 for a = 3 up to 96 atoms (12 000
 // genotypes of 45 atoms 176 -> 186, of 90 atoms 84.0 -> 86.4), 3 from 250
-// atoms on (256 x 8192 15.4 -> 16.8: a fourth block's shared memory leaves the
-// L1 cache 20 KB), else 4.
+// atoms on, where a fourth block's shared memory does not fit (256 atoms, 40
+// torsions, 8192 genotypes 15.4 -> 16.8) or leaves the L1 cache little (256
+// atoms, 20 torsions, 4000 genotypes 15.3 -> 15.8), else 4.  Four blocks an SM
+// that do not fit also run as 3 (256 atoms, 40 torsions, 1000 genotypes 10.4 ->
+// 11.5).
 template <int A, int VAR, int MB>
 __global__ void __launch_bounds__(128, MB) eval_ring_kernel(const RingArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -642,12 +645,14 @@ cudaError_t launch_ring_t(const RingArgs &a, int threads, int smem, cudaStream_t
     return cudaGetLastError();
 }
 
-// need: blocks an SM that hold the whole launch at once.
+// need: blocks an SM that hold the whole launch at once; fit: blocks whose
+// shared memory an SM holds.
 template <int A, int VAR>
-cudaError_t launch_ring_mb(const RingArgs &a, int need, int threads, int smem, cudaStream_t s) {
+cudaError_t launch_ring_mb(const RingArgs &a, int need, int fit, int threads, int smem,
+                           cudaStream_t s) {
     if constexpr (VAR == ADGB_REDUCE_SHFL) {
         if (need <= 2) return launch_ring_t<A, VAR, 2>(a, threads, smem, s);
-        if (need <= 3 || (need > 4 && a.lig.n_atoms >= 250))
+        if (need <= 3 || fit <= 3 || (need > 4 && a.lig.n_atoms >= 250))
             return launch_ring_t<A, VAR, 3>(a, threads, smem, s);
     }
     if constexpr (A == 3)
@@ -656,16 +661,16 @@ cudaError_t launch_ring_mb(const RingArgs &a, int need, int threads, int smem, c
 }
 
 template <int A>
-cudaError_t launch_ring_v(const RingArgs &a, int variant, int need, int threads, int smem,
+cudaError_t launch_ring_v(const RingArgs &a, int variant, int need, int fit, int threads, int smem,
                           cudaStream_t s) {
     switch (variant) {
-        case ADGB_REDUCE_SHFL: return launch_ring_mb<A, ADGB_REDUCE_SHFL>(a, need, threads, smem, s);
+        case ADGB_REDUCE_SHFL: return launch_ring_mb<A, ADGB_REDUCE_SHFL>(a, need, fit, threads, smem, s);
         case ADGB_REDUCE_MMA_TF32X2:
-            return launch_ring_mb<A, ADGB_REDUCE_MMA_TF32X2>(a, need, threads, smem, s);
+            return launch_ring_mb<A, ADGB_REDUCE_MMA_TF32X2>(a, need, fit, threads, smem, s);
         case ADGB_REDUCE_MMA_BF16X3:
-            return launch_ring_mb<A, ADGB_REDUCE_MMA_BF16X3>(a, need, threads, smem, s);
+            return launch_ring_mb<A, ADGB_REDUCE_MMA_BF16X3>(a, need, fit, threads, smem, s);
         case ADGB_REDUCE_TCGEN05:
-            return launch_ring_mb<A, ADGB_REDUCE_TCGEN05>(a, need, threads, smem, s);
+            return launch_ring_mb<A, ADGB_REDUCE_TCGEN05>(a, need, fit, threads, smem, s);
     }
     return cudaErrorInvalidValue;
 }
@@ -746,13 +751,16 @@ cudaError_t launch_eval_ring(const RecDev &rec, const LigDev &lig, const EvalCfg
     if (e != cudaSuccess) return e;
     const int smem = tc_smem_bytes(a.L.total, rs.warps, cfg.variant, dev);
     if (smem < 0) return cudaErrorInvalidValue;
-    int sms = 0;
+    int sms = 0, per_sm = 0, reserved = 0;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&per_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     if (e != cudaSuccess) return e;
+    const int fit = per_sm / (smem + reserved);
     const int need = ((n + 1) / 2 + sms - 1) / sms;
-    if (rs.a == 3) return launch_ring_v<3>(a, cfg.variant, need, 32 * rs.warps, smem, s);
-    if (rs.a == 4) return launch_ring_v<4>(a, cfg.variant, need, 32 * rs.warps, smem, s);
-    return launch_ring_v<5>(a, cfg.variant, need, 32 * rs.warps, smem, s);
+    if (rs.a == 3) return launch_ring_v<3>(a, cfg.variant, need, fit, 32 * rs.warps, smem, s);
+    if (rs.a == 4) return launch_ring_v<4>(a, cfg.variant, need, fit, 32 * rs.warps, smem, s);
+    return launch_ring_v<5>(a, cfg.variant, need, fit, 32 * rs.warps, smem, s);
 }
 
 cudaError_t ring_tc_gave_up_async(unsigned int *dst, cudaStream_t s) {
