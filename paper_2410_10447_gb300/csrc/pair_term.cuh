@@ -38,11 +38,14 @@ __device__ __forceinline__ float rcp_ftz(float x) {
 // function and no square root (its error, half an ulp of a b under the root,
 // that of rsqrt.approx and one rounding, is below that of sqrtf times
 // rsqrtf).  Where a b leaves the normal range, the two roots themselves.
+__device__ __forceinline__ float root_ratio(float a, float b) {
+    const float ab = __fmul_rn(a, b);
+    if (ab > 1e-36f && ab < 1e38f) return __fmul_rn(a, rsqrt_ftz(ab));
+    return __fmul_rn(sqrtf(a), rsqrtf(b));
+}
+// Of two genotypes, each by its own range: neither's bits depend on the other.
 __device__ __forceinline__ float2 root_ratio2(float2 a, float2 b) {
-    const float2 ab = mul2(a, b);
-    const bool fine = ab.x > 1e-36f && ab.x < 1e38f && ab.y > 1e-36f && ab.y < 1e38f;
-    if (fine) return mul2(a, make_float2(rsqrt_ftz(ab.x), rsqrt_ftz(ab.y)));
-    return make_float2(sqrtf(a.x) * rsqrtf(b.x), sqrtf(a.y) * rsqrtf(b.y));
+    return make_float2(root_ratio(a.x, b.x), root_ratio(a.y, b.y));
 }
 
 // Two pair terms from their squared distances r2 and constants A, B (12-6

@@ -220,3 +220,37 @@ def test_bits_do_not_depend_on_the_launch_size(pkg, torch, cfg1, variant):
         b, g, _ = ctx.local_search(rid, lid, genes, 8, variant=variant)
         assert np.array_equal(b[-8:], ref[0]) and np.array_equal(g[-8:], ref[1]), n
     ctx.close()
+
+
+@pytest.mark.parametrize("n_atoms", [32, 45])
+def test_range_of_the_adadelta_state_is_each_genotypes_own(pkg, torch, n_atoms):
+    """A running average outside the fast form's range (sums of squares whose
+    product overflows FP32) takes its own genotype to the general form, not
+    the one it is searched with: the same bits beside such a genotype, beside
+    an ordinary one and alone, in both two-genotypes kernels."""
+    rec = synth.make_receptor(synth.generate.BASE_SEED + 5, 48, 8)
+    lig = synth.make_ligand(51_000 + n_atoms, n_atoms, 8, 8)
+    genes = synth.make_poses(52_000 + n_atoms, 4, rec, lig["n_tors"])
+    G = genes.shape[1]
+    rng = np.random.default_rng(n_atoms)
+    state = np.empty((4, 3, G), np.float32)
+    state[:, 0] = genes
+    state[:, 1:] = rng.uniform(0.1, 2.0, (4, 2, G))
+    state[1::2, 1] *= np.float32(1e30)
+    state[1::2, 2] *= np.float32(1e20)
+    ctx = pkg.Context(0)
+    rid, lid = ctx.upload_receptor_grids(rec), ctx.upload_ligand_torsion_tree(lig)
+
+    def search(order):
+        b, g, st = ctx.local_search(rid, lid, genes[order].copy(), 3, state=state[order],
+                                    resume=True, want_state=True)
+        return b, g, st
+
+    ref = search([0, 1, 2, 3])
+    mixed = search([0, 2, 1, 3])
+    for a, m in zip(ref, mixed):
+        assert np.array_equal(a[[0, 2, 1, 3]], m)
+    for p in range(4):
+        for a, m in zip(ref, search([p])):
+            assert np.array_equal(a[p:p + 1], m), p
+    ctx.close()
