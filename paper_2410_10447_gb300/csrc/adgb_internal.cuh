@@ -231,6 +231,7 @@ __host__ __device__ inline bool pair_eligible(int n_atoms, int n_tors, int n_pai
 // la <= 32 lanes: as many as fit a warp, every team of every warp taking a
 // slice of the steps.  Larger la: the warps cover the lanes in windows of 32,
 // and sets of `windows` warps take slices of the steps.
+constexpr int RING_WARPS = 4;   // warps of a block
 struct RingShape {
     int a, la, np;        // atoms a lane, lanes, ring length
     int windows, teams;   // warps the lanes span; teams a warp
@@ -251,7 +252,7 @@ __host__ __device__ inline RingShape ring_shape(int N) {
     r.np = r.a * r.la;
     r.windows = (r.la + 31) / 32;
     r.teams = r.windows > 1 ? 1 : 32 / r.la;
-    r.warps = 4;
+    r.warps = RING_WARPS;
     r.slices = r.windows > 1 ? r.warps / r.windows : r.teams * r.warps;
     const int s = r.np / 2 + r.a - 1;
     r.steps = (s + r.slices - 1) / r.slices;
@@ -278,7 +279,7 @@ __host__ __device__ inline int ring_next(int j, int res) {
 __host__ __device__ inline int ring_entries(int len, int res) { return res ? 4 * res : len; }
 // Slice of the steps whose reactions copy c holds.
 __host__ __device__ inline int ring_slice(const RingShape &r, int c) {
-    return r.windows > 1 ? c / r.windows : c;
+    return r.windows > 1 ? c >> 1 : c;   // (two windows at most: 64 lanes)
 }
 // A lane's place: ring lane l, first step s0, force copy.
 struct RingLane {

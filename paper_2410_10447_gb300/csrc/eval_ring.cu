@@ -21,25 +21,30 @@
 // (26 packed and 14 scalar instructions for a pair of two genotypes, 15 more
 // for distances, sums and the reaction; 256 atoms: FMA pipe 50%, issue 46%,
 // LSU data pipe 31% busy, the rest fixed latencies at 10-15 warps an SM); below
-// that, the latency of an evaluation's seven barriers, torsion walk and grid
-// loads.  The kernel it took over from for these ligands (one genotype a 64-
+// that, the latency of an evaluation's six barriers, gene threads, torsion walk
+// and grid loads (45 atoms, one block an SM: ring 2300 of 6500 cycles, gene
+// threads 1000, walk 700, grid 700, torsions 950, atoms' sums 650).  The kernel it took over from for these ligands (one genotype a 64-
 // or 128-thread group, forces through per-pair slots in shared memory) had its
 // LSU data pipe 73% busy at 256 atoms, 46% of the shared-memory wavefronts
 // bank-conflict replays, at 107K warp instructions an evaluation; this one
 // issues 42K.  Local search, M evaluations/s before -> with the sweep:
-// 45 atoms x 1000 genotypes 95 -> 159, 64 x 8000 58 -> 121, 90 x 1500
-// 31 -> 85, 128 x 8000 17 -> 52, 192 x 6000 10 -> 28, 256 x 2048 6.2 -> 13.4,
-// x 8192 6.8 -> 15.5 (with 3 or 5 atoms a lane only, no 4: 64 x 8000 113,
-// 128 x 8000 43, 256 x 2048 12.1: idle lanes).
+// 45 atoms x 1000 genotypes 95 -> 157, 64 x 8000 58 -> 121, 90 x 1500
+// 31 -> 87, 128 x 8000 17 -> 53, 160 x 6000 12 -> 38, 256 x 2048 6.2 -> 16.0
+// (with 3 or 5 atoms a lane only, no 4, and then 4: 64 x 8000 113 -> 121, 128 x
+// 8000 43 -> 52, 256 x 2048 12.1 -> 13.4: idle lanes).  Two steps' pairs
+// computed before both reactions are stored, to overlap their chains: 2-5%
+// slower (registers).
 //
 // Per evaluation (block barriers between the steps):
-//   1. gene threads publish genes and sin / (1 - cos) of every angle;
+//   1. genes and sin / (1 - cos) of every angle are there (step 6, or the
+//      kernel's start, published them);
 //   2. a thread an atom and genotype: torsion walk, grid terms, and the sums
 //      of (E, g, torque) of the grid terms: pair forces are central and
 //      cancel in the rigid-body sums exactly, so they take no part in them;
 //   3. ring sweep; 4. atoms' total gradients;
 //   5. torsions' moving-set sums (8 lanes a torsion) and the reduction;
-//   6. gene gradient, best tracking and ADADELTA by the gene threads.
+//   6. gene gradient, best tracking, ADADELTA and the next angles' sines by
+//      the gene threads, a gene and genotype each.
 #include <math.h>
 
 #include <algorithm>
@@ -64,7 +69,7 @@ struct RingSmem {
     int cxy, cz;        // force copies [copies][copy_len], as the positions
     int gxy, gz;        // atoms' gradients [N], as the positions
     int genes, sc, ggrad, red, stage;
-    int ada;            // gene threads' state [MAX_GENES][4]: E[g^2], E[d^2], best, Omega
+    int ada;            // gene threads' state [MAX_GENES][genotype]: E[g^2], E[d^2], best, Omega
     int total;
     RingShape r;
 
@@ -159,7 +164,7 @@ __device__ __forceinline__ float reduce_parity8(float v[8]) {
 }
 
 // Whole evaluation loop of a block's two genotypes (all threads).
-template <int A, int VAR>
+template <int A, int VAR, bool AHEAD>
 __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L, const LigDev &lig,
                                             const RecDev &rec, const PairIO &io, Tc05Warp &tw) {
     const int t = threadIdx.x, TH = blockDim.x, lane = t & 31, warp = t >> 5;
@@ -184,38 +189,43 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
     float *red = reinterpret_cast<float *>(sm + L.red);   // [warp][genotype][8]
     float *stage = reinterpret_cast<float *>(sm + L.stage) + warp * 32 * 12;
 
-    // the thread's gene (j = t) of both genotypes, and ADADELTA state
-    const int j = t;
-    float2 om = bc(0.f), eg2 = bc(0.f), ed2 = bc(0.f);
-    if (j < G) {
-#pragma unroll
-        for (int g = 0; g < 2; g++) {
-            float o, a = 0.f, b = 0.f;
-            if (io.resume) {
-                const float *st = io.state[g];
-                o = st[j];
-                a = st[G + j];
-                b = st[2 * G + j];
-            } else {
-                o = io.genes_in[g][j];
-            }
-            if (g == 0) {
-                om.x = o; eg2.x = a; ed2.x = b;
-            } else {
-                om.y = o; eg2.y = a; ed2.y = b;
-            }
+    // Thread t < 2 G: gene jj of genotype gen and its ADADELTA state, kept in
+    // shared memory between evaluations (the ring sweep needs the registers).
+    // The thread that steps a gene also takes the sine and cosine of its angle
+    // and publishes them: one barrier an evaluation less than with a thread a
+    // gene for both genotypes, and with the sums over the warps unrolled
+    // (step 6) the gene threads' chain is 1450 -> 1000 of an evaluation's 7400
+    // cycles (45 atoms, one block an SM).
+    const int gen = t & 1;
+    const bool gene_thread = t < 2 * G;
+    const int jj = min(t >> 1, MAX_GENES - 1);
+    float4 *ada = reinterpret_cast<float4 *>(sm + L.ada) + 2 * jj + gen;   // E[g^2], E[d^2], best, Omega
+    // publishes the gene and sin / (1 - cos) of its angle (half-angle form:
+    // exact zero at a zero angle; phi and theta as (sin, cos) of the angle)
+    auto publish = [&](float om) {
+        const bool full = jj == 3 || jj == 4;
+        float sn, cs;
+        sincosf(full ? om : 0.5f * om, &sn, &cs);
+        reinterpret_cast<float *>(genes_s)[2 * jj + gen] = om;
+        const float2 w = full ? make_float2(sn, cs) : make_float2(2.f * sn * cs, 2.f * sn * sn);
+        float2 *sc2 = reinterpret_cast<float2 *>(sc) + gen;
+        if (jj >= 6) sc2[2 * (jj - 6)] = w;
+        else if (jj >= 3) sc2[2 * (SC_ROT + jj - 3)] = w;
+    };
+    if (gene_thread) {
+        float o, a = 0.f, b = 0.f;
+        if (io.resume) {
+            const float *st = io.state[gen];
+            o = st[jj];
+            a = st[G + jj];
+            b = st[2 * G + jj];
+        } else {
+            o = io.genes_in[gen][jj];
         }
+        *ada = make_float4(a, b, o, o);
+        publish(o);
     }
-    // (between evaluations it lives in shared memory: the ring sweep needs the
-    // registers)
-    float2 *ada = reinterpret_cast<float2 *>(sm + L.ada) + 4 * min(j, MAX_GENES - 1);
-    if (j < G) {
-        ada[0] = eg2;
-        ada[1] = ed2;
-        ada[2] = ada[3] = om;
-    }
-    __syncthreads();
-    float2 best_e = bc(INFINITY);
+    float best_e = INFINITY;
     // the lane's place in the ring sweep
     const RingLane rl = ring_lane(rs, warp, lane);
     const int copy_ent = ring_entries(rs.copy_len, rs.copy_res);
@@ -223,27 +233,10 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
     auto pos_at = [&](int q) { return ring_index<A>(q, rs.pos_res); };
     auto copy_at = [&](int q) { return ring_index<A>(q, rs.copy_res); };
     const float4 *table = lig.ring + (size_t)warp * rs.steps * A * 32 + lane;
-    // the thread's genotype in steps 2 and 5 (blockDim.x is even)
-    const int gen = t & 1;
     const int iters = max(io.iters[0], io.iters[1]);
 
     for (int it = 0; it < iters; it++) {
-        // 1. genes and sin / (1 - cos) of every angle, a thread a gene and
-        //    genotype (half-angle form: exact zero at a zero angle; phi and
-        //    theta as (sin, cos) of the angle)
-        if (t < 2 * G) {
-            const int jj = t >> 1;
-            const float om = reinterpret_cast<const float *>(sm + L.ada)[8 * jj + 6 + gen];
-            const bool full = jj == 3 || jj == 4;
-            float sn, cs;
-            sincosf(full ? om : 0.5f * om, &sn, &cs);
-            reinterpret_cast<float *>(genes_s)[2 * jj + gen] = om;
-            const float2 w = full ? make_float2(sn, cs) : make_float2(2.f * sn * cs, 2.f * sn * sn);
-            float2 *sc2 = reinterpret_cast<float2 *>(sc) + gen;
-            if (jj >= 6) sc2[2 * (jj - 6)] = w;
-            else if (jj >= 3) sc2[2 * (SC_ROT + jj - 3)] = w;
-        }
-        __syncthreads();
+        __syncthreads();   // 1. the genes and angles are published
 
         // 2. coordinates and grid terms of the thread's atoms in its genotype
         float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -319,7 +312,18 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
                 xi[a] = load_v2(pxy, pz, pos_at(A * rl.l + a));
                 fi[a] = {bc(0.f), bc(0.f), bc(0.f)};
             }
+            // AHEAD: the constants of the next step are loaded before this one's
+            // terms.  Taken where a block has 254 registers a thread (launches of
+            // up to two blocks an SM; 300 genotypes of 256 atoms 9.9 -> 10.6M
+            // evaluations/s, of 128 atoms 26.4 -> 27.8); with 168 or 128 the other
+            // resident blocks hide the loads (2048 x 256 atoms 15.8 -> 15.7, 6000
+            // x 160 37.2 -> 36.4).
             const float4 *tp = table;
+            float4 nc[A];
+            if constexpr (AHEAD) {
+#pragma unroll
+                for (int a = 0; a < A; a++) nc[a] = __ldg(tp + 32 * a);
+            }
             // atom a l + s0 + st of the ring and its place in the copy
             int pj = pos_at(A * rl.l + rl.s0), cj = copy0 + copy_at(A * rl.l);
 #pragma unroll 2
@@ -327,9 +331,17 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
                 const V2 xj = load_v2(pxy, pz, A == 4 ? pj : pj + st);
                 if constexpr (A == 4) pj += ring_next<A>(rl.s0 + st, rs.pos_res);
                 V2 fj = {bc(0.f), bc(0.f), bc(0.f)};
+                float4 cc[A];
+#pragma unroll
+                for (int a = 0; a < A; a++) cc[a] = AHEAD ? nc[a] : __ldg(tp + 32 * a);
+                if constexpr (AHEAD) {
+                    const float4 *tn = st + 1 < rs.steps ? tp + A * 32 : tp;
+#pragma unroll
+                    for (int a = 0; a < A; a++) nc[a] = __ldg(tn + 32 * a);
+                }
 #pragma unroll
                 for (int a = 0; a < A; a++) {
-                    const float4 pc = __ldg(tp + 32 * a);
+                    const float4 pc = cc[a];
                     const bool hb = __float_as_int(pc.x) < 0;
                     // x_i - x_j, exact; as FMAs 0.8% faster here than as adds
                     const float2 m1 = bc(-1.f);
@@ -373,15 +385,17 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
         if (lig.n_pairs > 0 && T > 0) {
             for (int i = t; i < N; i += TH) {
                 V2 g = load_v2(gxy, gz, i);
-#pragma unroll 4
-                for (int c = 0; c < rs.copies; c++) {
-                    int q = i - 1 - ring_slice(rs, c) * rs.steps;
-                    if (q < 0) q += rs.np;
-                    const V2 f = load_v2(cxy, cz, c * copy_ent + copy_at(q));
-                    g = {add2(g.x, f.x), add2(g.y, f.y), add2(g.z, f.z)};
-                    if (q + rs.np < rs.copy_len) {   // at most one more turn (copy_len < 2 np)
-                        const V2 h = load_v2(cxy, cz, c * copy_ent + copy_at(q + rs.np));
-                        g = {add2(g.x, h.x), add2(g.y, h.y), add2(g.z, h.z)};
+                for (int c0 = 0; c0 < rs.copies; c0 += RING_WARPS) {
+#pragma unroll
+                    for (int c = c0; c < c0 + RING_WARPS; c++) {
+                        int q = i - 1 - ring_slice(rs, c) * rs.steps;
+                        if (q < 0) q += rs.np;
+                        const V2 f = load_v2(cxy, cz, c * copy_ent + copy_at(q));
+                        g = {add2(g.x, f.x), add2(g.y, f.y), add2(g.z, f.z)};
+                        if (q + rs.np < rs.copy_len) {   // at most one more turn (copy_len < 2 np)
+                            const V2 h = load_v2(cxy, cz, c * copy_ent + copy_at(q + rs.np));
+                            g = {add2(g.x, h.x), add2(g.y, h.y), add2(g.z, h.z)};
+                        }
                     }
                 }
                 gxy[i] = make_float4(g.x.x, g.x.y, g.y.x, g.y.y);
@@ -400,6 +414,7 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
             if (k < T) {
                 ta = s_tat[k];
                 xb = load_v2(pxy, pz, pos_at(ta.y));
+#pragma unroll 1   // (unrolled 2 and 4 times: 1-3% slower)
                 for (int i = ta.z + (t & 7); i < ta.w; i += 8) {
                     const V2 g = load_v2(gxy, gz, i), x = load_v2(pxy, pz, pos_at(i));
                     const V2 d = {sub2(x.x, xb.x), sub2(x.y, xb.y), sub2(x.z, xb.z)};
@@ -453,102 +468,78 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
         }
         // what the gene formulas take from this evaluation's genes, read
         // before the barrier after which they may be rewritten
-        const float4 c_phi = sc[SC_ROT], c_th = sc[SC_ROT + 1], c_al = sc[SC_ROT + 2];
+        const float2 *sc_rot = reinterpret_cast<const float2 *>(sc) + 2 * SC_ROT + gen;
+        const float2 c_phi = sc_rot[0], c_th = sc_rot[2], c_al = sc_rot[4];
         __syncthreads();
 
-        // 6. gene gradient, best tracking, ADADELTA
-        if (j < G) {
+        // 6. gene gradient, best tracking, ADADELTA; the next evaluation's genes
+        if (gene_thread) {
             auto total = [&](int c) {
-                float2 s = make_float2(red[c], red[8 + c]);
-                for (int w = 1; w < rs.warps; w++)
-                    s = add2(s, make_float2(red[16 * w + c], red[16 * w + 8 + c]));
+                float s = red[8 * gen + c];
+#pragma unroll
+                for (int w = 1; w < RING_WARPS; w++) s = __fadd_rn(s, red[16 * w + 8 * gen + c]);
                 return s;
             };
-            const float2 E = total(0);
-            float2 gj;
-            if (j < 3) {
-                gj = total(1 + j);
-            } else if (j < 6) {
+            const float E = total(0);
+            float gj;
+            if (jj < 6) {
                 // d u / d phi or d theta; angular velocity sin(a) du + (1-cos a) u x du
-                const float2 sphi = make_float2(c_phi.x, c_phi.z), cphi = make_float2(c_phi.y, c_phi.w);
-                const float2 sth = make_float2(c_th.x, c_th.z), cth = make_float2(c_th.y, c_th.w);
-                const float2 s = make_float2(c_al.x, c_al.z), o = make_float2(c_al.y, c_al.w);
-                const V2 u = {mul2(sth, cphi), mul2(sth, sphi), cth};
-                const bool th = j == 4;
-                const V2 du = {th ? mul2(cth, cphi) : mul2(bc(-1.f), mul2(sth, sphi)),
-                               th ? mul2(cth, sphi) : mul2(sth, cphi),
-                               th ? mul2(bc(-1.f), sth) : bc(0.f)};
-                const V2 uxd = cross2(u, du);
-                const V2 wv = {fma2(s, du.x, mul2(o, uxd.x)), fma2(s, du.y, mul2(o, uxd.y)),
-                               fma2(s, du.z, mul2(o, uxd.z))};
-                const V2 tq = {total(4), total(5), total(6)};
-                gj = dot2(tq, j == 5 ? u : wv);
+                const float3 u = make_float3(c_th.x * c_phi.y, c_th.x * c_phi.x, c_th.y);
+                const bool th = jj == 4;
+                const float3 du = make_float3(th ? c_th.y * c_phi.y : -c_th.x * c_phi.x,
+                                              th ? c_th.y * c_phi.x : c_th.x * c_phi.y,
+                                              th ? -c_th.x : 0.f);
+                auto det = [](float p, float q, float r, float s) {   // p q - r s
+                    return __fmaf_rn(p, q, -__fmul_rn(r, s));
+                };
+                const float3 uxd = make_float3(det(u.y, du.z, u.z, du.y), det(u.z, du.x, u.x, du.z),
+                                               det(u.x, du.y, u.y, du.x));
+                const float3 w = make_float3(__fmaf_rn(c_al.x, du.x, __fmul_rn(c_al.y, uxd.x)),
+                                             __fmaf_rn(c_al.x, du.y, __fmul_rn(c_al.y, uxd.y)),
+                                             __fmaf_rn(c_al.x, du.z, __fmul_rn(c_al.y, uxd.z)));
+                const float3 d = jj == 5 ? u : w;
+                const float t0 = total(jj < 3 ? 1 + jj : 4);
+                gj = jj < 3 ? t0 : __fmaf_rn(total(6), d.z, __fmaf_rn(total(5), d.y, __fmul_rn(t0, d.x)));
             } else {
-                gj = ggrad[j];
+                gj = reinterpret_cast<const float *>(ggrad)[2 * jj + gen];
             }
             if (io.mode == MODE_SCORE) {
-                if (j == 0) {
-                    io.energy[0][0] = E.x;
-                    if (io.nvalid > 1) io.energy[1][0] = E.y;
+                if (gen < io.nvalid) {
+                    if (jj == 0) io.energy[gen][0] = E;
+                    if (io.grad[gen]) io.grad[gen][jj] = gj;
                 }
-                if (io.grad[0]) io.grad[0][j] = gj.x;
-                if (io.nvalid > 1 && io.grad[1]) io.grad[1][j] = gj.y;
             } else {
-                float2 eg2 = ada[0], ed2 = ada[1], om = ada[3];
-                const bool act_a = it < io.iters[0], act_b = it < io.iters[1];
-                if (act_a && E.x < best_e.x) {
-                    best_e.x = E.x;
-                    ada[2].x = om.x;
+                float4 a = *ada;
+                if (it < io.iters[gen]) {
+                    if (E < best_e) {
+                        best_e = E;
+                        a.z = a.w;
+                    }
+                    const float omr = 1.f - io.rho;
+                    a.x = __fmaf_rn(io.rho, a.x, __fmul_rn(omr, __fmul_rn(gj, gj)));
+                    const float d = __fmul_rn(
+                        root_ratio(__fadd_rn(a.y, io.eps), __fadd_rn(a.x, io.eps)), -gj);
+                    a.y = __fmaf_rn(io.rho, a.y, __fmul_rn(omr, __fmul_rn(d, d)));
+                    float w = __fadd_rn(a.w, d);
+                    if (jj >= 6) w -= 2.f * PI_F * floorf((w + PI_F) * (0.5f / PI_F));
+                    a.w = w;
+                    *ada = a;
+                    publish(w);
                 }
-                if (act_b && E.y < best_e.y) {
-                    best_e.y = E.y;
-                    ada[2].y = om.y;
-                }
-                const float2 rho = bc(io.rho), omr = bc(1.f - io.rho), ep = bc(io.eps);
-                const float2 neg2 = fma2(rho, eg2, mul2(omr, mul2(gj, gj)));
-                const float2 a2 = add2(ed2, ep), b2 = add2(neg2, ep);
-                const float2 d = mul2(root_ratio2(a2, b2), make_float2(-gj.x, -gj.y));
-                const float2 ned2 = fma2(rho, ed2, mul2(omr, mul2(d, d)));
-                float2 w = add2(om, d);
-                if (j >= 6) {
-                    w.x -= 2.f * PI_F * floorf((w.x + PI_F) * (0.5f / PI_F));
-                    w.y -= 2.f * PI_F * floorf((w.y + PI_F) * (0.5f / PI_F));
-                }
-                if (act_a) {
-                    eg2.x = neg2.x;
-                    ed2.x = ned2.x;
-                    om.x = w.x;
-                }
-                if (act_b) {
-                    eg2.y = neg2.y;
-                    ed2.y = ned2.y;
-                    om.y = w.y;
-                }
-                ada[0] = eg2;
-                ada[1] = ed2;
-                ada[3] = om;
             }
         }
         if (io.mode == MODE_SCORE) return;
-        __syncthreads();   // the updated genes are published by other threads
     }
-    if (io.mode == MODE_SCORE || j >= G) return;
-    const float2 best = ada[2];
-    eg2 = ada[0];
-    ed2 = ada[1];
-    om = ada[3];
-#pragma unroll
-    for (int g = 0; g < 2; g++) {
-        if (g >= io.nvalid) break;
-        io.genes_out[g][j] = g ? best.y : best.x;
-        if (io.state[g]) {
-            float *st = io.state[g];
-            st[j] = g ? om.y : om.x;
-            st[G + j] = g ? eg2.y : eg2.x;
-            st[2 * G + j] = g ? ed2.y : ed2.x;
-        }
-        if (j == 0) io.energy[g][0] = g ? best_e.y : best_e.x;
+    if (io.mode == MODE_SCORE || !gene_thread || gen >= io.nvalid) return;
+    const float4 a = *ada;
+    io.genes_out[gen][jj] = a.z;
+    if (io.state[gen]) {
+        float *st = io.state[gen];
+        st[jj] = a.w;
+        st[G + jj] = a.x;
+        st[2 * G + jj] = a.y;
     }
+    if (jj == 0) io.energy[gen][0] = best_e;
 }
 
 // Resident blocks of 128 threads an SM the kernels are built for (MB), i.e.
@@ -591,7 +582,7 @@ __global__ void __launch_bounds__(128, MB) eval_ring_kernel(const RingArgs a) {
     io.resume = a.resume;
     io.rho = a.rho;
     io.eps = a.eps;
-    search_ring<A, VAR>(sm, a.L, a.lig, a.rec, io, tw);
+    search_ring<A, VAR, MB == 2>(sm, a.L, a.lig, a.rec, io, tw);
     tc_end<VAR>(tw);
     if constexpr (VAR != ADGB_REDUCE_TCGEN05) dependents_may_start();
 }
@@ -630,7 +621,7 @@ __global__ void __launch_bounds__(128, 4) eval_ring_items_kernel(const WorkItem 
     io.resume = 0;
     io.rho = w.rho;
     io.eps = w.eps;
-    search_ring<A, VAR>(sm, L, lig, recs[w.rec], io, tw);
+    search_ring<A, VAR, false>(sm, L, lig, recs[w.rec], io, tw);
     tc_end<VAR>(tw);
 }
 
