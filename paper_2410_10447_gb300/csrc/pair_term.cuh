@@ -38,13 +38,18 @@ __device__ __forceinline__ float rcp_ftz(float x) {
 // function and no square root (its error, half an ulp of a b under the root,
 // that of rsqrt.approx and one rounding, is below that of sqrtf times
 // rsqrtf).  Where a b leaves the normal range, the two roots themselves.
+__device__ __forceinline__ bool root_ratio_fine(float ab) { return ab > 1e-36f && ab < 1e38f; }
 __device__ __forceinline__ float root_ratio(float a, float b) {
     const float ab = __fmul_rn(a, b);
-    if (ab > 1e-36f && ab < 1e38f) return __fmul_rn(a, rsqrt_ftz(ab));
+    if (root_ratio_fine(ab)) return __fmul_rn(a, rsqrt_ftz(ab));
     return __fmul_rn(sqrtf(a), rsqrtf(b));
 }
-// Of two genotypes, each by its own range: neither's bits depend on the other.
+// Of two genotypes, each by its own range (neither's bits depend on the
+// other); one branch where both are in range.
 __device__ __forceinline__ float2 root_ratio2(float2 a, float2 b) {
+    const float2 ab = mul2(a, b);
+    if (root_ratio_fine(ab.x) && root_ratio_fine(ab.y))
+        return mul2(a, make_float2(rsqrt_ftz(ab.x), rsqrt_ftz(ab.y)));
     return make_float2(root_ratio(a.x, b.x), root_ratio(a.y, b.y));
 }
 
