@@ -19,15 +19,15 @@
 //
 // What bounds it: from ~90 atoms on, the issue and FMA pipe of the pair terms
 // (26 packed and 14 scalar instructions for a pair of two genotypes, 15 more
-// for distances, sums and the reaction; 256 atoms: FMA pipe 50%, issue 46%,
-// LSU data pipe 31% busy, the rest fixed latencies at 10-15 warps an SM); below
+// for distances, sums and the reaction; 256 atoms: FMA pipe 52%, issue 47%,
+// LSU data pipe 37% busy, the rest fixed latencies at 10-15 warps an SM); below
 // that, the latency of an evaluation's six barriers, gene threads, torsion walk
 // and grid loads (45 atoms, one block an SM: ring 2300 of 6500 cycles, gene
 // threads 1000, walk 700, grid 700, torsions 950, atoms' sums 650).  The kernel it took over from for these ligands (one genotype a 64-
 // or 128-thread group, forces through per-pair slots in shared memory) had its
 // LSU data pipe 73% busy at 256 atoms, 46% of the shared-memory wavefronts
 // bank-conflict replays, at 107K warp instructions an evaluation; this one
-// issues 42K.  Local search, M evaluations/s before -> with the sweep:
+// issues 40K.  Local search, M evaluations/s before -> with the sweep:
 // 45 atoms x 1000 genotypes 95 -> 157, 64 x 8000 58 -> 121, 90 x 1500
 // 31 -> 87, 128 x 8000 17 -> 53, 160 x 6000 12 -> 38, 256 x 2048 6.2 -> 16.0
 // (with 3 or 5 atoms a lane only, no 4, and then 4: 64 x 8000 113 -> 121, 128 x
@@ -547,15 +547,15 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
 // spilled outside the sweep).  All give the same bits.  A launch that needs no
 // more blocks an SM takes the kernel with more registers, whose loads and pair
 // chains overlap better (M evaluations/s, shuffle form, 4 -> 3 -> 2 blocks;
-// 300 genotypes, one block an SM: 45 atoms 60 -> 64 -> 64, 90 33 -> 37 -> 39,
-// 160 14 -> 16 -> 21, 256 - -> 7.9 -> 10.0; 900 genotypes, three: 45 atoms 148
-// -> 155, 160 30 -> 33).  Larger launches: 5 for a = 3 up to 96 atoms (12 000
-// genotypes of 45 atoms 176 -> 186, of 90 atoms 84.0 -> 86.4), 3 from 250
-// atoms on, where a fourth block's shared memory does not fit (256 atoms, 40
-// torsions, 8192 genotypes 15.4 -> 16.8) or leaves the L1 cache little (256
-// atoms, 20 torsions, 4000 genotypes 15.3 -> 15.8), else 4.  Four blocks an SM
-// that do not fit also run as 3 (256 atoms, 40 torsions, 1000 genotypes 10.4 ->
-// 11.5).
+// 300 genotypes, one block an SM: 45 atoms 70 -> 73 -> 74, 90 36 -> 40 -> 41,
+// 160 16 -> 18 -> 22, 256 7.0 -> 9.0 -> 10.7; 900 genotypes, three, 4 -> 3: 45
+// atoms 160 -> 166, 160 32 -> 34).  Larger launches: 5 for a = 3 up to 96 atoms
+// (12 000 genotypes of 45 atoms 206 -> 214, of 90 atoms 91.8 -> 92.4), 3 from
+// 250 atoms on, where a fourth block's shared memory does not fit (256 atoms,
+// 40 torsions, 8192 genotypes 15.9 -> 17.7) or leaves the L1 cache little (256
+// atoms, 20 torsions, 4000 genotypes 15.8 -> 16.7), else 4 (128 atoms, 8000
+// genotypes, 3 -> 4: 52.5 -> 53.2).  Four blocks an SM that do not fit also run
+// as 3 (256 atoms, 40 torsions, 1000 genotypes 10.6 -> 12.5).
 template <int A, int VAR, int MB>
 __global__ void __launch_bounds__(128, MB) eval_ring_kernel(const RingArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
