@@ -411,6 +411,8 @@ int rescore_fp64_dev(adgb_ctx *ctx, int receptor_id, int ligand_id, const float 
  * stragglers; a context with a launch shape of its own runs one persistent
  * launch over all items.  The launches are captured into a CUDA graph on the
  * first call and replayed by later calls with the same buffers and parameters.
+ * A call with others may come while earlier ones still run (the third such
+ * call in a row waits on the host for the first).
  *
  * batch_create - item i: n_poses[i] genotypes of ligand ligand_ids[i]
  *   against receptor receptor_ids[i].  Genotypes of item i occupy rows

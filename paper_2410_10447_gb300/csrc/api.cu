@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <list>
 #include <map>
 #include <string>
 #include <vector>
@@ -32,6 +33,13 @@ struct Ligand {
 }  // namespace
 
 namespace {
+// Kinds of launches a batch may need: one a class of ring shapes (a = 3, 4 or
+// 5), two genotypes a warp, one genotype a warp.
+constexpr int BATCH_CLASSES = 5;
+// Plans a batch rotates through, so that a call with other buffers need not
+// wait for the call before it.
+constexpr size_t BATCH_PLANS = 2;
+
 // An uneven batch: items of (receptor, ligand, genotype count) run by one
 // persistent multi-ligand launch replayed from a captured CUDA graph.
 struct ItemClass {
@@ -40,6 +48,31 @@ struct ItemClass {
     int first, count;       // its items
     int cost, budget, grid; // largest item, layout bytes, persistent blocks
 };
+// The work items of one set of buffers and parameters on the device, and the
+// graph that runs them.  A launch reads the items as its blocks start, so a
+// plan is rewritten only after its latest launch has finished.
+struct BatchPlan {
+    WorkItem *items = nullptr;
+    int cap = 0;
+    int *counter = nullptr;          // [2 BATCH_CLASSES], re-armed by the kernels
+    std::vector<ItemClass> classes;
+    cudaGraphExec_t exec = nullptr;
+    cudaEvent_t done = nullptr;      // after the latest launch
+    long long launched = 0;          // its number among the batch's launches (0: none)
+};
+void drop_graph(BatchPlan &p) {
+    if (p.exec) cudaGraphExecDestroy(p.exec);
+    p.exec = nullptr;
+}
+
+void free_plan(BatchPlan &p) {
+    drop_graph(p);
+    if (p.done) cudaEventDestroy(p.done);
+    cudaFree(p.items);
+    cudaFree(p.counter);
+    p = BatchPlan();
+}
+
 struct Batch {
     std::vector<int> rec_idx, lig_idx, n_poses;  // per item, indices into the tables
     std::vector<LigDev> ligs;                    // unique ligands
@@ -48,13 +81,11 @@ struct Batch {
     long long total = 0;
     LigDev *d_ligs = nullptr;
     RecDev *d_recs = nullptr;
-    int *d_counter = nullptr;                    // [2], re-armed by the kernel
-    WorkItem *d_items = nullptr;
-    int items_cap = 0;
-    std::vector<ItemClass> classes;  // of the uploaded items
+    std::list<BatchPlan> plans;                  // up to BATCH_PLANS
+    BatchPlan *cur = nullptr;                    // the plan of the k_ fields, or null
+    long long launches = 0;
     EvalCfg cfg{32, 4, 0, 1, 0};
     bool tuned = false;
-    cudaGraphExec_t exec = nullptr;
     // what the captured graph was built for
     const float *k_genes = nullptr;
     const float *k_energy = nullptr;
@@ -62,10 +93,6 @@ struct Batch {
     float k_rho = 0.f, k_eps = 0.f;
 };
 }  // namespace
-
-// Kinds of launches a batch may need: one a class of ring shapes (a = 3, 4 or
-// 5), two genotypes a warp, one genotype a warp.
-constexpr int BATCH_CLASSES = 5;
 
 struct adgb_ctx {
     int device = 0;
@@ -1052,11 +1079,9 @@ int adgb_destroy(adgb_ctx *c) {
         DeviceGuard g(c->device);
         for (auto &kv : c->batches) {
             Batch &b = kv.second;
-            if (b.exec) cudaGraphExecDestroy(b.exec);
+            for (BatchPlan &p : b.plans) free_plan(p);
             cudaFree(b.d_ligs);
             cudaFree(b.d_recs);
-            cudaFree(b.d_counter);
-            cudaFree(b.d_items);
         }
         for (auto &kv : c->recs) cudaFree(kv.second.cells);
         for (auto &kv : c->ligs) cudaFree(kv.second.mem);
@@ -1835,23 +1860,56 @@ std::vector<WorkItem> batch_items(const Batch &b, const EvalCfg &cfg, float *gen
     return out;
 }
 
-cudaError_t upload_items(Batch &b, const std::vector<WorkItem> &items, cudaStream_t s) {
-    if ((int)items.size() > b.items_cap) {
-        if (b.d_items) cudaFree(b.d_items);
-        b.d_items = nullptr;
-        cudaError_t e = cudaMalloc(&b.d_items, sizeof(WorkItem) * std::max<size_t>(items.size(), 1));
-        if (e != cudaSuccess) return e;
-        b.items_cap = (int)items.size();
+// A plan of the batch that may be rewritten: one whose launches have
+// finished, else a new one, else the one launched longest ago (the host waits
+// for it).
+cudaError_t take_plan(Batch &b, BatchPlan **out) {
+    BatchPlan *pick = nullptr;
+    bool finished = false;
+    for (BatchPlan &p : b.plans) {
+        const cudaError_t q = p.launched ? cudaEventQuery(p.done) : cudaSuccess;
+        if (q == cudaErrorNotReady) (void)cudaGetLastError();   // not a later launch's error
+        else if (q != cudaSuccess) return q;
+        finished = q == cudaSuccess;
+        if (finished || !pick || p.launched < pick->launched) pick = &p;
+        if (finished) break;
     }
-    cudaError_t e = cudaMemcpyAsync(b.d_items, items.data(), sizeof(WorkItem) * items.size(),
-                                    cudaMemcpyHostToDevice, s);
+    if (!finished && b.plans.size() < BATCH_PLANS) {
+        b.plans.emplace_back();
+        pick = &b.plans.back();
+    } else if (!finished) {
+        const cudaError_t e = cudaEventSynchronize(pick->done);
+        if (e != cudaSuccess) return e;
+    }
+    if (b.cur == pick) b.cur = nullptr;
+    drop_graph(*pick);
+    *out = pick;
+    return cudaSuccess;
+}
+
+cudaError_t upload_items(BatchPlan &p, const std::vector<WorkItem> &items, cudaStream_t s) {
+    cudaError_t e = cudaSuccess;
+    if (!p.counter) {
+        e = cudaMalloc(&p.counter, 2 * BATCH_CLASSES * sizeof(int));
+        if (e == cudaSuccess) e = cudaMemsetAsync(p.counter, 0, 2 * BATCH_CLASSES * sizeof(int), s);
+        if (e != cudaSuccess) return e;
+    }
+    if (!p.done && (e = cudaEventCreateWithFlags(&p.done, cudaEventDisableTiming)) != cudaSuccess) return e;
+    if ((int)items.size() > p.cap) {
+        cudaFree(p.items);
+        p.items = nullptr;
+        p.cap = 0;
+        if ((e = cudaMalloc(&p.items, sizeof(WorkItem) * std::max<size_t>(items.size(), 1))) != cudaSuccess) return e;
+        p.cap = (int)items.size();
+    }
+    e = cudaMemcpyAsync(p.items, items.data(), sizeof(WorkItem) * items.size(), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     return e;
 }
 
 // Persistent grids of the classes that use one; false if a shape fits no SM.
-bool batch_grids(Batch &b, int device) {
-    for (ItemClass &k : b.classes) {
+bool batch_grids(BatchPlan &p, int device) {
+    for (ItemClass &k : p.classes) {
         if (k.ring_a) continue;
         k.grid = items_grid(k.cfg, k.budget, device);
         if (k.grid < 1) return false;
@@ -1859,11 +1917,11 @@ bool batch_grids(Batch &b, int device) {
     return true;
 }
 
-// Launches every class of the batch's uploaded items, the first on `s`, the
+// Launches every class of the plan's uploaded items, the first on `s`, the
 // others on the context's side streams between a fork and a join on `s`, so
 // that a class's last blocks overlap with the next class's first.
-cudaError_t launch_batch(adgb_ctx *c, Batch &b, cudaStream_t s) {
-    const int n = (int)b.classes.size();
+cudaError_t launch_batch(adgb_ctx *c, const Batch &b, const BatchPlan &p, cudaStream_t s) {
+    const int n = (int)p.classes.size();
     cudaError_t e = cudaSuccess;
     if (n > 1) {
         if (!c->fork) e = cudaEventCreateWithFlags(&c->fork, cudaEventDisableTiming);
@@ -1875,14 +1933,14 @@ cudaError_t launch_batch(adgb_ctx *c, Batch &b, cudaStream_t s) {
         if (e == cudaSuccess) e = cudaEventRecord(c->fork, s);
     }
     for (int q = 0; q < n && e == cudaSuccess; q++) {
-        const ItemClass &k = b.classes[q];
+        const ItemClass &k = p.classes[q];
         const cudaStream_t t = q == 0 ? s : c->side[q - 1];
         if (q > 0) e = cudaStreamWaitEvent(t, c->fork, 0);
         if (e != cudaSuccess) break;
-        const WorkItem *items = b.d_items + k.first;
+        const WorkItem *items = p.items + k.first;
         e = k.ring_a ? launch_eval_ring_items(items, k.count, b.d_ligs, b.d_recs, k.ring_a,
                                               k.ring_warps, k.budget, k.cfg.variant, t)
-                     : launch_eval_items(items, k.count, b.d_ligs, b.d_recs, b.d_counter + 2 * q,
+                     : launch_eval_items(items, k.count, b.d_ligs, b.d_recs, p.counter + 2 * q,
                                          k.cfg, k.budget, k.grid, t);
         if (q > 0) {   // join also after a failed launch, so that a capture can end
             cudaError_t j = cudaEventRecord(c->join[q - 1], t);
@@ -1936,14 +1994,11 @@ extern "C" int batch_create(adgb_ctx *c, int n_items, const int *receptor_ids, c
     DeviceGuard g(c->device);
     cudaError_t e = cudaMalloc(&b.d_ligs, sizeof(LigDev) * b.ligs.size());
     if (e == cudaSuccess) e = cudaMalloc(&b.d_recs, sizeof(RecDev) * b.recs.size());
-    if (e == cudaSuccess) e = cudaMalloc(&b.d_counter, 2 * BATCH_CLASSES * sizeof(int));
     if (e == cudaSuccess) e = cudaMemcpy(b.d_ligs, b.ligs.data(), sizeof(LigDev) * b.ligs.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(b.d_recs, b.recs.data(), sizeof(RecDev) * b.recs.size(), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(b.d_counter, 0, 2 * BATCH_CLASSES * sizeof(int));
     if (e != cudaSuccess) {
         cudaFree(b.d_ligs);
         cudaFree(b.d_recs);
-        cudaFree(b.d_counter);
         return fail(c, ADGB_ENOMEM, "batch_create: %s", cudaGetErrorString(e));
     }
     b.cfg.variant = c->opts.reduce_variant;
@@ -1971,11 +2026,9 @@ extern "C" int batch_release(adgb_ctx *c, int batch_id) {
     if (it == c->batches.end()) return fail(c, ADGB_ENOTFOUND, "unknown batch id %d", batch_id);
     DeviceGuard g(c->device);
     Batch &b = it->second;
-    if (b.exec) cudaGraphExecDestroy(b.exec);
+    for (BatchPlan &p : b.plans) free_plan(p);
     cudaFree(b.d_ligs);
     cudaFree(b.d_recs);
-    cudaFree(b.d_counter);
-    cudaFree(b.d_items);
     c->batches.erase(it);
     return ADGB_OK;
 }
@@ -1998,27 +2051,28 @@ extern "C" int batch_local_search_dev(adgb_ctx *c, int batch_id, float *genes_de
     cfg.paired = cfg.paired && batch_pairable(b, cfg);
     cfg.ring = cfg.ring && batch_ringable(b);
     cudaError_t e = cudaSuccess;
-    const bool same = b.exec && b.k_genes == genes_dev && b.k_energy == best_energy_dev &&
+    const bool same = b.cur && b.k_genes == genes_dev && b.k_energy == best_energy_dev &&
                       b.k_iters == p->iters && b.k_rho == p->rho && b.k_eps == p->eps &&
                       b.k_tpp == cfg.tpp && b.k_ppb == cfg.ppb && b.k_var == cfg.variant &&
                       b.k_paired == cfg.paired && b.k_ring == cfg.ring;
     if (!same) {
-        if (b.exec) cudaGraphExecDestroy(b.exec);
-        b.exec = nullptr;
+        BatchPlan *plan = nullptr;
+        if ((e = take_plan(b, &plan)) != cudaSuccess) return cuda_fail(c, e, "batch_local_search");
         const std::vector<WorkItem> items =
-            batch_items(b, cfg, genes_dev, best_energy_dev, p->iters, p->rho, p->eps, b.classes);
-        if (!batch_grids(b, c->device)) return fail(c, ADGB_EINVAL, "batch_local_search: launch shape does not fit an SM");
-        e = upload_items(b, items, c->stream);
+            batch_items(b, cfg, genes_dev, best_energy_dev, p->iters, p->rho, p->eps, plan->classes);
+        if (!batch_grids(*plan, c->device)) return fail(c, ADGB_EINVAL, "batch_local_search: launch shape does not fit an SM");
+        e = upload_items(*plan, items, c->stream);
         cudaGraph_t graph = nullptr;
         if (e == cudaSuccess) e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            const cudaError_t el = launch_batch(c, b, c->stream);
+            const cudaError_t el = launch_batch(c, b, *plan, c->stream);
             e = cudaStreamEndCapture(c->stream, &graph);
             if (el != cudaSuccess) e = el;
         }
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&b.exec, graph, 0);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&plan->exec, graph, 0);
         if (graph) cudaGraphDestroy(graph);
         if (e != cudaSuccess) return cuda_fail(c, e, "batch_local_search: graph capture");
+        b.cur = plan;
         b.k_genes = genes_dev;
         b.k_energy = best_energy_dev;
         b.k_iters = p->iters;
@@ -2030,7 +2084,11 @@ extern "C" int batch_local_search_dev(adgb_ctx *c, int batch_id, float *genes_de
         b.k_paired = cfg.paired;
         b.k_ring = cfg.ring;
     }
-    e = cudaGraphLaunch(b.exec, (cudaStream_t)stream);
+    e = cudaGraphLaunch(b.cur->exec, (cudaStream_t)stream);
+    if (e == cudaSuccess) {
+        b.cur->launched = ++b.launches;
+        e = cudaEventRecord(b.cur->done, (cudaStream_t)stream);
+    }
     return e == cudaSuccess ? ADGB_OK : cuda_fail(c, e, "batch_local_search: graph launch");
 }
 
@@ -2064,18 +2122,20 @@ extern "C" int batch_autotune(adgb_ctx *c, int batch_id, const float *genes_dev,
     if (e == cudaSuccess) e = cudaMalloc(&te, sizeof(float) * (size_t)b.total);
     if (e == cudaSuccess) e = cudaEventCreate(&e0);
     if (e == cudaSuccess) e = cudaEventCreate(&e1);
+    BatchPlan *plan = nullptr;
+    if (e == cudaSuccess) e = take_plan(b, &plan);
     float best_ms = INFINITY;
     EvalCfg best{};
     for (const EvalCfg &cfg : cands) {
         if (e != cudaSuccess) break;
-        const std::vector<WorkItem> items = batch_items(b, cfg, tg, te, iters, 0.8f, 1e-2f, b.classes);
-        if (!batch_grids(b, c->device)) continue;
+        const std::vector<WorkItem> items = batch_items(b, cfg, tg, te, iters, 0.8f, 1e-2f, plan->classes);
+        if (!batch_grids(*plan, c->device)) continue;
         float ms_min = INFINITY;
         for (int rep = 0; rep < 2 && e == cudaSuccess; rep++) {
             e = cudaMemcpyAsync(tg, genes_dev, gbytes, cudaMemcpyDeviceToDevice, c->stream);
-            if (e == cudaSuccess && rep == 0) e = upload_items(b, items, c->stream);
+            if (e == cudaSuccess && rep == 0) e = upload_items(*plan, items, c->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e0, c->stream);
-            if (e == cudaSuccess) e = launch_batch(c, b, c->stream);
+            if (e == cudaSuccess) e = launch_batch(c, b, *plan, c->stream);
             if (e == cudaSuccess) e = cudaEventRecord(e1, c->stream);
             if (e == cudaSuccess) e = cudaEventSynchronize(e1);
             float ms = 0.f;
@@ -2095,10 +2155,7 @@ extern "C" int batch_autotune(adgb_ctx *c, int batch_id, const float *genes_dev,
     if (!(best_ms < INFINITY)) return fail(c, ADGB_EINVAL, "batch_autotune: no launch shape fits");
     b.cfg = best;
     b.tuned = true;
-    if (b.exec) {
-        cudaGraphExecDestroy(b.exec);
-        b.exec = nullptr;
-    }
+    b.cur = nullptr;
     c->tune_table[tune_key(b)] = best;
     if (chosen) {
         chosen->threads_per_pose = best.tpp;

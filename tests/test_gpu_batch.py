@@ -142,3 +142,32 @@ def test_uneven_512_full_size_sampled(pkg, torch):
             assert be[row] <= e0 + max(1e-4 * abs(e0), 1e-3)
     ctx.batch_release(bid)
     ctx.close()
+
+
+def test_batch_calls_with_other_buffers_back_to_back(pkg, torch):
+    """Several waves of blocks, other buffers in every call, no
+    synchronisation between the calls: each returns what it returns alone."""
+    rec = synth.make_receptor(synth.generate.BASE_SEED + 3, 48, 6)
+    ligs = [synth.make_ligand(500 + a, a, 6, 6) for a in (20, 40, 60, 90)]
+    n = 400                                   # 600 blocks and more of each ligand class
+    ctx = pkg.Context(0)
+    rid = ctx.upload_receptor_grids(rec)
+    bid = ctx.batch_create([rid] * 4, [ctx.upload_ligand_torsion_tree(L) for L in ligs], [n] * 4)
+    starts = [torch.from_numpy(pack([synth.make_poses(600 + 10 * c + i, n, rec, 6) for i in range(4)])).cuda()
+              for c in range(4)]
+
+    def calls(wait):
+        genes, energy = [s.clone() for s in starts], [torch.zeros(4 * n, device="cuda") for _ in starts]
+        torch.cuda.synchronize()
+        for c, (g, e) in enumerate(zip(genes, energy)):
+            ctx.batch_local_search_dev(bid, g, e, 20 + c)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return genes, energy
+
+    alone, together = calls(True), calls(False)
+    for x, y in zip(alone[0] + alone[1], together[0] + together[1]):
+        assert torch.equal(x, y)
+    ctx.batch_release(bid)
+    ctx.close()
