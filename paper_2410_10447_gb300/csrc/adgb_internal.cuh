@@ -214,6 +214,9 @@ struct PairSmem {
     }
 };
 
+// Genotypes of a block of the two-genotypes kernels at most (two warps).
+constexpr int PAIR_MAX_PPB = 4;
+
 // Whether a ligand runs two genotypes a warp: at most 32 atoms with the
 // warp form of the matching rounds (or no pairs), at most 32 genes (one gene
 // slot a lane), one warp a genotype.

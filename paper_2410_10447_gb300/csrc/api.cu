@@ -1776,6 +1776,7 @@ EvalCfg item_cfg(const LigDev &l, const EvalCfg &cfg, int *ring_a, int *ring_war
     *ring_a = *ring_warps = 0;
     EvalCfg e = cfg;
     e.ring = 0;
+    if (e.paired) e.ppb = std::min(e.ppb, PAIR_MAX_PPB);   // what a block of that kernel searches
     if (!cfg.ring) return e;
     e.tpp = 32;
     e.ppb = 4;
@@ -2107,8 +2108,7 @@ extern "C" int batch_autotune(adgb_ctx *c, int batch_id, const float *genes_dev,
                            {32, 4, ADGB_REDUCE_MMA_BF16X3, 1, 0, 0}, {32, 4, ADGB_REDUCE_TCGEN05, 1, 0, 0},
                            {32, 2, ADGB_REDUCE_SHFL, 1, 0, 0}, {64, 2, ADGB_REDUCE_SHFL, 1, 0, 0},
                            {128, 1, ADGB_REDUCE_SHFL, 1, 0, 0},
-                           {32, 4, ADGB_REDUCE_SHFL, 1, 0, 1}, {32, 8, ADGB_REDUCE_SHFL, 1, 0, 1},
-                           {32, 4, ADGB_REDUCE_TCGEN05, 1, 0, 1}, {32, 8, ADGB_REDUCE_TCGEN05, 1, 0, 1},
+                           {32, 4, ADGB_REDUCE_SHFL, 1, 0, 1}, {32, 4, ADGB_REDUCE_TCGEN05, 1, 0, 1},
                            {128, 2, ADGB_REDUCE_SHFL, 1, 0, 0, 1}, {128, 2, ADGB_REDUCE_TCGEN05, 1, 0, 0, 1}};
     std::vector<EvalCfg> cands;
     for (const EvalCfg &cf : all)

@@ -35,6 +35,8 @@
 //   6. gene gradient, best tracking and ADADELTA by the gene lanes.
 #include <math.h>
 
+#include <algorithm>
+
 #include "adgb_internal.cuh"
 #include "packed.cuh"
 #include "pair_term.cuh"
@@ -977,7 +979,7 @@ cudaError_t launch_pair_items_t(const PairItemsArgs &a, int smem, int grid, cuda
 // genotypes a block (items header included).
 int pair_layout_bytes(int n_atoms, int n_tors, int ppb, int variant) {
     PairSmem L;
-    ppb = ppb < 1 ? 1 : (ppb > 4 ? 4 : ppb);
+    ppb = std::clamp(ppb, 1, PAIR_MAX_PPB);
     L.make(n_atoms, n_tors, (ppb + 1) / 2, variant != ADGB_REDUCE_TCGEN05);
     return L.total + PAIR_HDR;
 }
@@ -991,7 +993,7 @@ cudaError_t launch_eval_pair_items(const WorkItem *items, int n_items, const Lig
     a.recs = recs;
     a.counter = counter;
     a.n_items = n_items;
-    a.ppb = cfg.ppb < 1 ? 1 : (cfg.ppb > 4 ? 4 : cfg.ppb);
+    a.ppb = std::clamp(cfg.ppb, 1, PAIR_MAX_PPB);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -1008,7 +1010,7 @@ cudaError_t launch_eval_pair_items(const WorkItem *items, int n_items, const Lig
 
 // Resident blocks of a persistent paired launch: SMs x blocks an SM holds.
 int pair_items_grid(const EvalCfg &cfg, int budget, int device) {
-    const int ppb = cfg.ppb < 1 ? 1 : (cfg.ppb > 4 ? 4 : cfg.ppb);
+    const int ppb = std::clamp(cfg.ppb, 1, PAIR_MAX_PPB);
     const int threads = 32 * ((ppb + 1) / 2);
     const int smem = pair_smem_bytes(budget, threads / 32, cfg.variant, device);
     if (smem < 0) return 0;
@@ -1095,7 +1097,7 @@ static cudaError_t launch_pair_any(const RecDev &rec, const LigDev &lig, const E
     PairArgs a;
     a.rec = rec;
     a.lig = lig;
-    a.ppb = cfg.ppb < 1 ? 1 : (cfg.ppb > 4 ? 4 : cfg.ppb);
+    a.ppb = std::clamp(cfg.ppb, 1, PAIR_MAX_PPB);
     const int warps = (a.ppb + 1) / 2;
     a.L.make(lig.n_atoms, lig.n_tors, warps, cfg.variant != ADGB_REDUCE_TCGEN05);
     a.genes_in = genes_in;

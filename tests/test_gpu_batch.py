@@ -171,3 +171,28 @@ def test_batch_calls_with_other_buffers_back_to_back(pkg, torch):
         assert torch.equal(x, y)
     ctx.batch_release(bid)
     ctx.close()
+
+
+@pytest.mark.parametrize("variant", [0, 3])
+@pytest.mark.parametrize("ppb", [1, 3, 5, 8])
+def test_batch_of_small_ligands_searches_every_genotype(pkg, torch, ppb, variant):
+    """Two genotypes a warp with any number of genotypes a block: a block of
+    that kernel holds at most four."""
+    rec = synth.make_receptor(synth.generate.BASE_SEED + 4, 40, 6)
+    ligs = [synth.make_ligand(700 + a, a, 6, 4) for a in (12, 24, 32)]
+    n_poses = [17, 9, 8]
+    genes = [synth.make_poses(710 + i, n, rec, L["n_tors"]) for i, (L, n) in enumerate(zip(ligs, n_poses))]
+    ctx = pkg.Context(0, threads_per_pose=32, poses_per_block=ppb)
+    rid = ctx.upload_receptor_grids(rec)
+    lids = [ctx.upload_ligand_torsion_tree(L) for L in ligs]
+    bid = ctx.batch_create([rid] * 3, lids, n_poses)
+    g = torch.from_numpy(pack(genes)).cuda()
+    e = torch.full((sum(n_poses),), float("nan"), device="cuda")
+    ctx.batch_local_search_dev(bid, g, e, 12, variant=variant)
+    r = 0
+    for lid, x in zip(lids, genes):
+        best, y, _ = ctx.local_search(rid, lid, x.copy(), 12, variant=variant)
+        assert np.array_equal(e.cpu().numpy()[r:r + len(x)], best)
+        assert np.array_equal(g.cpu().numpy()[r:r + len(x), :x.shape[1]], y)
+        r += len(x)
+    ctx.close()
