@@ -418,10 +418,25 @@ inline cudaError_t launch_dependent(void (*k)(P...), int grid, int block, int sm
 
 // Dynamic shared memory a launch may take without asking for more.
 constexpr int SMEM_DEFAULT_LIMIT = 46 * 1024;   // of 48 KB, static shared memory included
+// Lets kernel k launch with smem bytes.  The limit belongs to the kernel on
+// its device and is shared by every host thread and context, so it is only
+// ever set to the most that the device grants: set to one launch's bytes, it
+// could take away what another thread had just set for a larger launch of the
+// same kernel.  Occupancy follows a launch's own bytes, not the limit
+// (Solis-Wets, 24 to 128 atoms, 64 to 6000 genotypes: times within 1% with the
+// limit at the launch's bytes, at the most, or left alone).
 template <typename K>
 inline cudaError_t allow_smem(K k, int smem) {
     if (smem <= SMEM_DEFAULT_LIMIT) return cudaSuccess;
-    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    int dev = 0, most = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k);
+    if (e != cudaSuccess) return e;
+    most -= (int)fa.sharedSizeBytes;
+    if (smem > most) return cudaErrorInvalidValue;
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
 }
 
 // Host-side launchers (eval.cu, reduce_bench.cu).

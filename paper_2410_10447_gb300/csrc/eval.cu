@@ -1160,8 +1160,7 @@ int items_grid(const EvalCfg &cfg, int budget, int device) {
     cudaError_t e = cudaErrorInvalidValue;
 #define ADGB_OCC(TPP, VAR)                                                                   \
     if (cfg.tpp == TPP && cfg.variant == VAR) {                                              \
-        e = cudaFuncSetAttribute(eval_items_kernel<TPP, VAR>,                                \
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem);         \
+        e = allow_smem(eval_items_kernel<TPP, VAR>, smem);                                   \
         if (e == cudaSuccess && VAR == ADGB_REDUCE_TCGEN05) {                                \
             cudaFuncAttributes fa;                                                           \
             e = cudaFuncGetAttributes(&fa, eval_items_kernel<TPP, VAR>);                     \

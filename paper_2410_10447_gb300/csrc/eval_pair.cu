@@ -940,7 +940,7 @@ __global__ void __launch_bounds__(64, 5) eval_pair_items_kernel(const PairItemsA
 template <int VAR>
 cudaError_t pair_items_occupancy(int threads, int smem, int device, int *per_sm) {
     auto k = eval_pair_items_kernel<VAR>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     if (VAR != ADGB_REDUCE_TCGEN05)
         return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, k, threads, smem);

@@ -296,7 +296,7 @@ static cudaError_t launch_r(const float *in, int threads, int n_blocks, int reps
                             cudaStream_t s) {
     const int smem = (256 + (threads / 32) * 32 * 12) * 4;
     auto k = reduce4_kernel<VAR>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     k<<<n_blocks, threads, smem, s>>>(reinterpret_cast<const float4 *>(in),
                                       reinterpret_cast<float4 *>(out), reps, 0.f);
@@ -329,7 +329,7 @@ static cudaError_t launch_tc(const float *in, int threads, int n_blocks, int rep
     const int floor_smem = sm_smem / (fit + 1) - reserved + 16;
     if (smem < floor_smem) smem = floor_smem;
     auto k = reduce4_tc05_kernel<NG>;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = allow_smem(k, smem);
     if (e != cudaSuccess) return e;
     k<<<n_blocks, threads, smem, s>>>(reinterpret_cast<const float4 *>(in),
                                       reinterpret_cast<float4 *>(out), reps, 0.f,

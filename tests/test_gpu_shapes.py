@@ -72,3 +72,37 @@ def test_shape_parity(pkg, torch, rec, n_atoms, n_tors, pair_rounds):
     for p, (er, _, _, _) in enumerate(refs):
         assert abs(e1[p] - er) <= max(1e-4 * abs(er), 1e-3)
     ctx.close()
+
+
+def test_threads_with_different_shared_memory(pkg):
+    """Host threads that launch one kernel with different amounts of shared
+    memory above the default limit (ligands of 225 and 256 atoms: 50 and 58 KB)
+    do not refuse each other's launches."""
+    import threading
+    import torch
+    rec = synth.make_receptor(synth.generate.BASE_SEED + 5, 40, 4)
+    errors, start = [], threading.Barrier(2)
+
+    def score(n_atoms, n_tors, variant):
+        try:
+            ctx = pkg.Context(0)
+            rid = ctx.upload_receptor_grids(rec)
+            lid = ctx.upload_ligand_torsion_tree(synth.make_ligand(800 + n_atoms, n_atoms, 4, n_tors))
+            genes = torch.from_numpy(synth.make_poses(801, 4, rec, n_tors)).cuda()
+            energy = torch.empty(4, device="cuda")
+            start.wait()
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(3000):
+                    ctx.score_poses_dev(rid, lid, genes, energy, None, variant)
+            torch.cuda.synchronize()
+            ctx.close()
+        except Exception as e:   # reported by the test's thread
+            errors.append(e)
+            start.abort()
+
+    threads = [threading.Thread(target=score, args=a) for a in ((225, 12, 0), (256, 40, 0))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
