@@ -80,51 +80,66 @@ __device__ void block_argmin(float e, int k, float *s_e, int *s_k, float &best_e
     __syncthreads();
 }
 
-// One GA generation: a warp an individual.  A child's random words are the
+// One GA generation: LANES lanes an individual.  A child's random words are the
 // Philox blocks 0 (tournaments), 1 (crossover, cuts, local search) and
-// 2 + j / 2 (gene j's mutation), at most 25: every lane computes one of them
-// and the words go round by shuffles, so a child costs one Philox call's
-// latency.  (A thread an individual ran two calls a gene in sequence, with a
-// run's 150 individuals on one SM: 10.2 us a generation of 20 x 150
-// individuals of 14 genes, now 5.1.)
-constexpr int GA_WARPS = 8;
-__global__ void __launch_bounds__(32 * GA_WARPS) ga_kernel(int n_runs, int pop, int G, const float *go,
-                                                           const float *eo, const DockCfg d,
-                                                           uint32_t gen, float *gn, int *iters,
-                                                           const int *done) {
+// 2 + j / 2 (gene j's mutation), at most 25: lane l computes blocks l, l +
+// LANES, .. (BL of them) and the words go round by shuffles.  A warp an
+// individual while all individuals' warps fit the GPU at once: a child costs
+// one Philox call's latency.  (A thread an individual ran two calls a gene in
+// sequence, with a run's 150 individuals on one SM: 20 x 150 individuals of 14
+// genes 9.3 us a generation, now 4.7.)  Above that the instructions of 32 lanes
+// are what takes the time, and 8 lanes compute 1, 2 or 4 blocks each: 300 x 150
+// individuals of 14 genes 10.8 us with a thread an individual, 16.0 with a
+// warp, 9.1 with 8 lanes; 1000 x 1000 119, 319 and 138 (of 46 genes 371, 389
+// and 293); 100 x 1000 18.9, 34.3 and 19.2, with 4 lanes 22 (the lanes of one
+// individual seek the run's best).
+constexpr int GA_THREADS = 256;
+template <int LANES, int BL>
+__global__ void __launch_bounds__(GA_THREADS) ga_kernel(int n_runs, int pop, int G, const float *go,
+                                                        const float *eo, const DockCfg d,
+                                                        uint32_t gen, float *gn, int *iters,
+                                                        const int *done) {
     wait_for_predecessor();
-    const int idx = blockIdx.x * GA_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int idx = blockIdx.x * (GA_THREADS / LANES) + threadIdx.x / LANES;
+    const int lane = threadIdx.x & (LANES - 1);
+    // the individual's lanes, which shuffle among themselves (of the warp's
+    // other individuals some may have returned or run another branch)
+    const unsigned group = LANES == 32 ? 0xffffffffu
+                                       : ((1u << LANES) - 1) << (threadIdx.x & 31 & ~(LANES - 1));
     if (idx >= n_runs * pop) return;
     const int run = idx / pop, k = idx - run * pop;
     const size_t base = (size_t)run * pop;
     float *child = gn + (size_t)idx * G;
     if (done && done[run] != 0) {   // a stopped run keeps its population
         const float *src = go + (size_t)idx * G;
-        for (int j = lane; j < G; j += 32) child[j] = src[j];
+        for (int j = lane; j < G; j += LANES) child[j] = src[j];
         if (lane == 0) iters[idx] = 0;
         return;
     }
-    const Philox4 o = philox4x32_10((uint32_t)k, gen, (uint32_t)run, (uint32_t)lane,
-                                    (uint32_t)d.seed, (uint32_t)(d.seed >> 32));
-    auto word = [&](int w) {   // word w (the same in every lane) of the child's stream
-        const uint32_t x = (w & 2) ? ((w & 1) ? o.w : o.z) : ((w & 1) ? o.y : o.x);
-        return __shfl_sync(0xffffffffu, x, w >> 2);
+    Philox4 o[BL];
+#pragma unroll
+    for (int b = 0; b < BL; b++)
+        o[b] = philox4x32_10((uint32_t)k, gen, (uint32_t)run, (uint32_t)(lane + LANES * b),
+                             (uint32_t)d.seed, (uint32_t)(d.seed >> 32));
+    auto word = [&](int w) {   // word w of blocks 0 and 1 (the same in every lane)
+        const uint32_t x = (w & 2) ? ((w & 1) ? o[0].w : o[0].z) : ((w & 1) ? o[0].y : o[0].x);
+        return __shfl_sync(group, x, w >> 2, LANES);
     };
     const uint32_t w_ls = word(W_LS);
     if (lane == 0) iters[idx] = unit24(w_ls) < d.ls_rate ? d.ls_iters : 1;
     if (k == 0) {   // the previous generation's best
         float e = INFINITY;
         int kk = 0x7fffffff;
-        for (int i = lane; i < pop; i += 32) {
+        for (int i = lane; i < pop; i += LANES) {
             const float v = eo[base + i];
             if (v < e || (v == e && i < kk)) {
                 e = v;
                 kk = i;
             }
         }
-        for (int off = 16; off > 0; off >>= 1) {
-            const float oe = __shfl_xor_sync(0xffffffffu, e, off);
-            const int ok = __shfl_xor_sync(0xffffffffu, kk, off);
+        for (int off = LANES / 2; off > 0; off >>= 1) {
+            const float oe = __shfl_xor_sync(group, e, off);
+            const int ok = __shfl_xor_sync(group, kk, off);
             if (oe < e || (oe == e && ok < kk)) {
                 e = oe;
                 kk = ok;
@@ -132,7 +147,7 @@ __global__ void __launch_bounds__(32 * GA_WARPS) ga_kernel(int n_runs, int pop, 
         }
         const int bk = kk < 0 || kk >= pop ? 0 : kk;
         const float *src = go + (base + bk) * G;
-        for (int j = lane; j < G; j += 32) child[j] = src[j];
+        for (int j = lane; j < G; j += LANES) child[j] = src[j];
         return;
     }
     int par[2];
@@ -151,11 +166,18 @@ __global__ void __launch_bounds__(32 * GA_WARPS) ga_kernel(int n_runs, int pop, 
         c1 = c2;
         c2 = t;
     }
-    for (int j0 = 0; j0 < G; j0 += 32) {
-        const int j = j0 + lane, src = (W_MUT + 2 * j) >> 2;   // lane of gene j's block
+    for (int j0 = 0; j0 < G; j0 += LANES) {
+        // genes j0 .. j0 + LANES - 1 read blocks b0 .. b0 + LANES / 2 - 1: of
+        // them, the lane holds at most one
+        const int j = j0 + lane, src = (W_MUT + 2 * j) >> 2, b0 = (W_MUT + 2 * j0) >> 2;
+        const int mine = (b0 + ((lane - b0) & (LANES - 1))) / LANES;
+        Philox4 m = o[0];
+#pragma unroll
+        for (int b = 1; b < BL; b++)
+            if (mine == b) m = o[b];
         const bool odd = j & 1;
-        const uint32_t mx = __shfl_sync(0xffffffffu, o.x, src & 31), my = __shfl_sync(0xffffffffu, o.y, src & 31);
-        const uint32_t mz = __shfl_sync(0xffffffffu, o.z, src & 31), mw = __shfl_sync(0xffffffffu, o.w, src & 31);
+        const uint32_t mx = __shfl_sync(group, m.x, src, LANES), my = __shfl_sync(group, m.y, src, LANES);
+        const uint32_t mz = __shfl_sync(group, m.z, src, LANES), mw = __shfl_sync(group, m.w, src, LANES);
         if (j < G) {
             float v = (j >= c1 && j < c2) ? B[j] : A[j];
             if (unit24(odd ? mz : mx) < d.p_mut) {
@@ -167,13 +189,31 @@ __global__ void __launch_bounds__(32 * GA_WARPS) ga_kernel(int n_runs, int pop, 
         }
     }
 }
-static_assert(((8 + 2 * (MAX_GENES - 1)) >> 2) < 32, "a child's Philox blocks exceed a warp");
+// Philox blocks of a child of G genes.
+constexpr int ga_blocks(int G) { return ((W_MUT + 2 * (G - 1) + 1) >> 2) + 1; }
+static_assert(ga_blocks(MAX_GENES) <= 32, "a child's Philox blocks exceed a warp");
+
+template <int LANES, int BL>
+cudaError_t launch_ga(const DockCfg &d, int G, int gen, const float *genes, const float *energy,
+                      float *genes_out, int *iters, const int *done, cudaStream_t s) {
+    const int n = d.n_runs * d.pop, per = GA_THREADS / LANES;
+    return launch_dependent(ga_kernel<LANES, BL>, (n + per - 1) / per, GA_THREADS, 0, s, d.n_runs, d.pop, G,
+                            genes, energy, d, (uint32_t)gen, genes_out, iters, done);
+}
 
 cudaError_t run_ga_kernel(const DockCfg &d, int G, int gen, const float *genes, const float *energy,
-                   float *genes_out, int *iters, const int *done, cudaStream_t s) {
-    const int n = d.n_runs * d.pop;
-    return launch_dependent(ga_kernel, (n + GA_WARPS - 1) / GA_WARPS, 32 * GA_WARPS, 0, s, d.n_runs,
-                            d.pop, G, genes, energy, d, (uint32_t)gen, genes_out, iters, done);
+                          float *genes_out, int *iters, const int *done, cudaStream_t s) {
+    int dev = 0, sms = 0, threads = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev);
+    if (e != cudaSuccess) return e;
+    const bool fits = (long long)d.n_runs * d.pop * 32 <= (long long)sms * threads;
+    const int blocks = ga_blocks(G);
+    if (fits) return launch_ga<32, 1>(d, G, gen, genes, energy, genes_out, iters, done, s);
+    if (blocks <= 8) return launch_ga<8, 1>(d, G, gen, genes, energy, genes_out, iters, done, s);
+    if (blocks <= 16) return launch_ga<8, 2>(d, G, gen, genes, energy, genes_out, iters, done, s);
+    return launch_ga<8, 4>(d, G, gen, genes, energy, genes_out, iters, done, s);
 }
 
 // A run evaluated in this pass (runs stopped before it have all iters 0).

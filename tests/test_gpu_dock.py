@@ -327,3 +327,34 @@ def test_dock_edge_sizes(pkg, torch, w):
         with pytest.raises(pkg.AdgbError):
             ctx.dock(rid, lid, pkg.adgb.dock_params(n_runs=1, pop=pop, max_gens=1, seed=1))
     ctx.close()
+
+
+@pytest.mark.parametrize("n_tors", [0, 6, 7, 22, 23, 40])
+def test_ga_generation_does_not_depend_on_the_launch_size(pkg, torch, n_tors):
+    """A launch of more individuals than the GPU holds warps gives each 8 lanes
+    with 1, 2 or 4 blocks of random words a lane (by the genes, edges at 12 and
+    28): the same children as of a launch of a few, a warp each."""
+    lig = synth.make_ligand(2600 + n_tors, max(8, 4 * n_tors + 8), 4, n_tors)
+    assert lig["n_tors"] == n_tors
+    G, pop, few = 6 + n_tors, 50, 3
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    runs = sms * 64 // pop + few
+    ctx = pkg.Context(0)
+    lid = ctx.upload_ligand_torsion_tree(lig)
+    gen = torch.Generator(device="cuda").manual_seed(n_tors)
+    genes = torch.empty(runs * pop, G, device="cuda").uniform_(-3, 3, generator=gen)
+    energy = torch.empty(runs * pop, device="cuda").normal_(generator=gen)
+    energy[::7] = energy[3]      # ties
+
+    def generation(n):
+        out, iters = torch.empty(n * pop, G, device="cuda"), torch.zeros(n * pop, dtype=torch.int32, device="cuda")
+        p = pkg.adgb.dock_params(n_runs=n, pop=pop, max_gens=3, ls_rate=0.3, seed=9)
+        ctx.ga_generation_dev(lid, p, 2, genes[:n * pop].contiguous(), energy[:n * pop].contiguous(), out, iters)
+        return out.cpu().numpy(), iters.cpu().numpy()
+
+    (a, ia), (b, ib) = generation(few), generation(runs)
+    assert np.array_equal(a, b[:few * pop]) and np.array_equal(ia, ib[:few * pop])
+    e = energy.cpu().numpy().reshape(runs, pop)
+    first = b.reshape(runs, pop, G)[:, 0]        # every run's best is kept
+    assert np.array_equal(first, genes.cpu().numpy().reshape(runs, pop, G)[np.arange(runs), e.argmin(1)])
+    ctx.close()
