@@ -759,13 +759,17 @@ __device__ __forceinline__ void search_pose_sw(unsigned char *sm, const SmemLayo
             float3 gi;
             e_part += inter_atom(rec, s_type[i], r4.w, x, gi);
         }
-        if (TPP == 32 && lig.r_lanes == 32 && lig.n_rounds > 0 && 64 * lig.n_rounds <= 3 * NP) {
+        if (TPP == 32 && VAR == ADGB_REDUCE_SHFL && lig.r_lanes == 32 && lig.n_rounds > 0 &&
+            64 * lig.n_rounds <= 3 * NP) {
             // matching rounds, two at a time: the partner's position by shuffles
             // and coalesced constants (from the pair list, four 16-byte loads of
             // random atoms for two pairs kept the LSU data pipe 70% busy).  Where
-            // two thirds of the rounds' lanes have a pair: 32 atoms (364 pairs,
-            // 11 rounds) 266 -> 242 us for 3000 genotypes x 60 evaluations, 24
-            // (186, 8) 206 -> 199; 16 (57, 5), the other side, 157 -> 169.
+            // two thirds of the rounds' lanes have a pair: 32 atoms (293 pairs,
+            // 10 rounds) 197 -> 170 us for 3000 genotypes x 40 evaluations, 24
+            // (161, 7) 160 -> 143; 16 (70, 5), the other side, 113 -> 126.  Not
+            // with the tensor-core reductions, whose chain has no room for the
+            // shuffles: 1500 genotypes of 32 atoms 193 -> 214 (tcgen05), 1000 of
+            // 28 atoms 125 -> 134 (TF32x2).
             const uint32_t *rw = lig.rword + gt;
             const float4 *rc = lig.rconst + gt;
             auto partner = [&](uint32_t w) {
@@ -792,19 +796,36 @@ __device__ __forceinline__ void search_pose_sw(unsigned char *sm, const SmemLayo
             }
         } else {
             group_sync<TPP>(group);
+            auto two = [&](uint32_t pa, uint32_t pb, float4 ka, float4 kb) {   // packed arithmetic
+                float3 fa, fb;
+                return pair_term2(xyz3(xyz[pa & 255]), xyz3(xyz[pb & 255]), xyz3(xyz[(pa >> 8) & 255]),
+                                  xyz3(xyz[(pb >> 8) & 255]), ka, kb, (pa >> 24) & 1, (pb >> 24) & 1, fa,
+                                  fb);
+            };
             int p = gt;
-            float3 fa, fb;
-            for (; p + TPP < NP; p += 2 * TPP) {  // pairs p and p + TPP, packed arithmetic
-                const uint32_t pa = prs[p], pb = prs[p + TPP];
-                e_part += pair_term2(xyz3(xyz[pa & 255]), xyz3(xyz[pb & 255]),
-                                     xyz3(xyz[(pa >> 8) & 255]), xyz3(xyz[(pb >> 8) & 255]),
-                                     __ldg(pconst + p), __ldg(pconst + p + TPP), (pa >> 24) & 1,
-                                     (pb >> 24) & 1, fa, fb);
+            // Two packed pairs at once, loaded together and added in the list's
+            // order: one at a time, a pass over the list took the latency of
+            // its loads and special functions every two pairs (3000 genotypes x
+            // 40 evaluations: 45 atoms 460 -> 451 us, 90 atoms 1190 -> 1146, 56
+            // atoms with tcgen05 929 -> 843; 64 genotypes of 80 atoms 193 -> 153,
+            // of 128 atoms 386 -> 269).  Where the rounds take the long lists,
+            // only short ones come here and the registers are needed there.
+            if constexpr (TPP > 32 || VAR != ADGB_REDUCE_SHFL) {
+                for (; p + 3 * TPP < NP; p += 4 * TPP) {
+                    const uint32_t pa = prs[p], pb = prs[p + TPP], pc = prs[p + 2 * TPP], pd = prs[p + 3 * TPP];
+                    const float4 ka = __ldg(pconst + p), kb = __ldg(pconst + p + TPP);
+                    const float4 kc = __ldg(pconst + p + 2 * TPP), kd = __ldg(pconst + p + 3 * TPP);
+                    const float e = two(pa, pb, ka, kb), e2 = two(pc, pd, kc, kd);
+                    e_part = (e_part + e) + e2;
+                }
             }
+            for (; p + TPP < NP; p += 2 * TPP)
+                e_part += two(prs[p], prs[p + TPP], __ldg(pconst + p), __ldg(pconst + p + TPP));
             if (p < NP) {
                 const uint32_t pr = prs[p];
+                float3 f;
                 e_part += pair_term(xyz[pr & 255], xyz[(pr >> 8) & 255], __ldg(pconst + p),
-                                    (pr >> 24) & 1, fa);
+                                    (pr >> 24) & 1, f);
             }
         }
         if constexpr (VAR == ADGB_REDUCE_SHFL) {   // one value: a butterfly
