@@ -88,8 +88,9 @@ typedef struct {
                               arithmetic in packed FP32x2 instructions - a warp for ligands of
                               at most 32 atoms (with matching rounds, at most 26 torsions, one
                               warp a genotype's atoms), a block (ring sweep of the pairs) for
-                              larger ones where neither threads_per_pose nor poses_per_block
-                              nor pair_rounds asks for another form; 1: one genotype a warp or
+                              larger ones that list enough of their pairs (about an eighth or
+                              more) where neither threads_per_pose nor poses_per_block nor
+                              pair_rounds asks for another form; 1: one genotype a warp or
                               group of warps */
 } adgb_options;
 
@@ -405,8 +406,8 @@ int rescore_fp64_dev(adgb_ctx *ctx, int receptor_id, int ligand_id, const float 
  * Uneven batches: genotypes of many ligands (of different atom, torsion and
  * pair counts), each against its own receptor, locally searched by one
  * multi-ligand call.  Every kind of ligand the batch holds (up to 32 atoms;
- * larger ones by the ring sweep's 3, 4 or 5 atoms a lane) is one launch over
- * its work items (a few genotypes of one ligand, longest first), and the
+ * larger ones by the ring sweep's 3, 4 or 5 atoms a lane, or with few pairs by
+ * the threads of a genotype) is one launch over its work items (a few genotypes of one ligand, longest first), and the
  * launches run side by side, so big and small ligands share the GPU without
  * stragglers; a context with a launch shape of its own runs one persistent
  * launch over all items.  The launches are captured into a CUDA graph on the

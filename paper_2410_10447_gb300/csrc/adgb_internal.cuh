@@ -345,6 +345,7 @@ struct EvalCfg {
     int stage_pairs;  // copy the pair list and incidence lists to shared memory
     int paired;     // two genotypes a warp where the ligand is eligible (pair_eligible)
     int ring;       // ring sweep, two genotypes a block, where the ligand has its table
+                    // (of a batch: every ligand in its own form)
 };
 
 // Carveout hint for the two-genotypes-a-warp kernels of the shuffle and

@@ -34,8 +34,8 @@ struct Ligand {
 
 namespace {
 // Kinds of launches a batch may need: one a class of ring shapes (a = 3, 4 or
-// 5), two genotypes a warp, one genotype a warp.
-constexpr int BATCH_CLASSES = 5;
+// 5), two genotypes a warp, one genotype in 32, 64 or 128 threads.
+constexpr int BATCH_CLASSES = 7;
 // Plans a batch rotates through, so that a call with other buffers need not
 // wait for the call before it.
 constexpr size_t BATCH_PLANS = 2;
@@ -435,6 +435,27 @@ void build_rounds(HostLigand &h) {
     }
 }
 
+// Whether the ring sweep takes a ligand of more than 32 atoms.  It computes
+// every pair of the ring, listed or not, so its time does not depend on the
+// list, while the force buffer's grows with the listed pairs and that of the
+// block form of the matching rounds (above 128 atoms) with the rounds.  The
+// lines are where both take the same time (lists thinned at random, 60, 1000
+// and 6000 genotypes), as a share of the ring table's slots: up to 48 atoms
+// 0.03-0.13 of them listed; 49-128 atoms 0.14-0.23 for 1000 and 6000
+// genotypes, 0.23-0.31 for 60 (up to 56 atoms less); rounds times lanes above
+// 128 atoms 0.15-0.20 up to 160 atoms, 0.25-0.30 at 192 to 256.  Ligands of one
+// or two torsions have such lists: 128 atoms, 728 pairs of 8704 slots, 1000
+// genotypes x 20 evaluations 421 us in the ring, 307 in the buffer; 112 atoms,
+// 108 of 7680, 382 and 213.  Without pairs the sweep is skipped.
+bool ring_pays(const HostLigand &h) {
+    if (h.NP == 0) return true;
+    const RingShape r = ring_shape(h.N);
+    const long long slots = (long long)r.warps * r.steps * r.a * 32;
+    if (h.N <= 48) return 10LL * h.NP >= slots;
+    if (h.N <= 128 || h.R == 0) return 4LL * h.NP >= slots;
+    return 10LL * h.R * h.VP >= 3 * slots;
+}
+
 // Pair constants in the order of the ring sweep (RingShape): a pair listed
 // more than once has its constants added (the pair term is linear in them).
 void build_ring(HostLigand &h) {
@@ -812,8 +833,9 @@ EvalCfg adgb::launch_cfg(const LigDev &L, int tpp_opt, int ppb_opt, int variant,
     cfg.ppb = ppb;
     cfg.paired = genotypes_per_warp == 0 &&
                  pair_eligible(L.n_atoms, L.n_tors, L.n_pairs, L.n_rounds, L.r_lanes, cfg.tpp);
-    // above 32 atoms the ring sweep, two genotypes a block, unless the caller
-    // set a launch shape or asked for one genotype a warp
+    // above 32 atoms the ring sweep, two genotypes a block, where the ligand has
+    // its table, unless the caller set a launch shape or asked for one genotype
+    // a warp
     cfg.ring = genotypes_per_warp == 0 && tpp_opt == 0 && ppb_opt == 0 && L.ring_n > 0;
     return cfg;
 }
@@ -868,9 +890,9 @@ int make_ligand_blob(std::string *err, const adgb_ligand_desc *d, int pair_round
     const size_t o_incoff = take(4 * (size_t)(NCH > 0 ? NCH : 1) * (N + 1)), o_inc = take(2 * 2 * (size_t)NPz);
     const size_t RVz = h.R > 0 ? (size_t)h.R * h.VP : 1;
     const size_t o_rword = take(4 * RVz), o_rconst = take(16 * RVz);
-    // the ring sweep: every ligand above 32 atoms, unless the caller asked for
-    // the force buffer
-    if (N >= RING_MIN_ATOMS && pair_rounds == 0) build_ring(h);
+    // the ring sweep: ligands above 32 atoms with enough pairs for it, unless
+    // the caller asked for the force buffer
+    if (N >= RING_MIN_ATOMS && pair_rounds == 0 && ring_pays(h)) build_ring(h);
     const size_t o_ring = take(16 * std::max<size_t>(h.ring.size(), 1));
     const size_t o_tR = take(4 * NT), o_teps = take(4 * NT), o_tvol = take(4 * NT),
                  o_tsol = take(4 * NT), o_thb = take(4 * NT);
@@ -1755,40 +1777,51 @@ extern "C" int dock_noalloc_dev(adgb_ctx *c, int receptor_id, int ligand_id,
 // ---------------------------------------------------------------------------
 namespace {
 
+bool own_forms(const adgb_ctx *c) { return c->opts.genotypes_per_warp == 0 && c->opts.pair_rounds == 0; }
+
 // Two genotypes a warp only when every ligand of the batch qualifies (one
-// launch shape serves the whole batch, unless the ring sweep is on).
+// launch shape serves the whole batch, unless each runs in its own form).
 bool batch_pairable(const Batch &b, const EvalCfg &cfg) {
     for (const LigDev &l : b.ligs)
         if (!pair_eligible(l.n_atoms, l.n_tors, l.n_pairs, l.n_rounds, l.r_lanes, cfg.tpp)) return false;
     return true;
 }
 
-// Whether any ligand of the batch has a ring table (the ring sweep then runs
-// those, and the smaller ones run two genotypes a warp where they qualify).
-bool batch_ringable(const Batch &b) {
+// Whether any ligand of the batch has more than 32 atoms (every ligand then
+// runs in its own form, if the batch's shape says so: cfg.ring).
+bool batch_has_large(const Batch &b) {
     for (const LigDev &l : b.ligs)
-        if (l.ring_n > 0) return true;
+        if (l.n_atoms >= RING_MIN_ATOMS) return true;
     return false;
 }
 
-// Launch shape of a ligand in a batch of shape cfg, and its ring class.
+// Launch shape of a ligand in a batch of shape cfg, and its ring class.  In
+// its own form: the ring sweep where it has a table, two genotypes a warp
+// where it qualifies, else one genotype in 64 threads up to 80 atoms (32
+// ligands of 57-80 atoms and one torsion, 64 genotypes each, 20 evaluations:
+// 290 us with 32 threads, 279 with 64, 355 with 128), in 128 above (of 90-128
+// atoms 1234, 1215 and 771).  A single call runs 57-80 atoms in 128 threads,
+// which take 1.27 times as long in a full GPU, so the ring starts at more
+// pairs here (the same 32 ligands with the single call's line 373 us).
 EvalCfg item_cfg(const LigDev &l, const EvalCfg &cfg, int *ring_a, int *ring_warps) {
     *ring_a = *ring_warps = 0;
     EvalCfg e = cfg;
     e.ring = 0;
-    if (e.paired) e.ppb = std::min(e.ppb, PAIR_MAX_PPB);   // what a block of that kernel searches
-    if (!cfg.ring) return e;
-    e.tpp = 32;
-    e.ppb = 4;
-    e.paired = pair_eligible(l.n_atoms, l.n_tors, l.n_pairs, l.n_rounds, l.r_lanes, 32);
-    if (l.ring_n > 0) {
-        const RingShape r = ring_shape(l.n_atoms);
-        e.ring = 1;
-        e.paired = 0;
-        e.ppb = 2;
-        *ring_a = r.a;
-        *ring_warps = r.warps;
+    if (cfg.ring) {
+        e.tpp = l.n_atoms < RING_MIN_ATOMS ? 32 : l.n_atoms <= 80 ? 64 : 128;
+        e.ppb = 128 / e.tpp;
+        e.paired = pair_eligible(l.n_atoms, l.n_tors, l.n_pairs, l.n_rounds, l.r_lanes, e.tpp);
+        const bool thin = l.n_atoms > 56 && l.n_atoms <= 80 && l.n_pairs > 0 && 20LL * l.n_pairs < 7LL * l.ring_n;
+        if (l.ring_n > 0 && !thin) {
+            const RingShape r = ring_shape(l.n_atoms);
+            e.ring = 1;
+            e.paired = 0;
+            e.ppb = 2;
+            *ring_a = r.a;
+            *ring_warps = r.warps;
+        }
     }
+    if (e.paired) e.ppb = std::min(e.ppb, PAIR_MAX_PPB);   // what a block of that kernel searches
     return e;
 }
 
@@ -1804,7 +1837,7 @@ std::vector<WorkItem> batch_items(const Batch &b, const EvalCfg &cfg, float *gen
         size_t q = 0;
         while (q < classes.size() &&
                !(classes[q].ring_a == k.ring_a && classes[q].ring_warps == k.ring_warps &&
-                 classes[q].cfg.paired == k.cfg.paired))
+                 (k.ring_a || (classes[q].cfg.paired == k.cfg.paired && classes[q].cfg.tpp == k.cfg.tpp))))
             q++;
         if (q == classes.size()) classes.push_back(k);
         cls[u] = (int)q;
@@ -2004,8 +2037,8 @@ extern "C" int batch_create(adgb_ctx *c, int n_items, const int *receptor_ids, c
     }
     b.cfg.variant = c->opts.reduce_variant;
     b.cfg.paired = c->opts.genotypes_per_warp == 0;
-    // the ring sweep unless the context set a launch shape
-    b.cfg.ring = b.cfg.paired && c->opts.threads_per_pose == 0 && c->opts.poses_per_block == 0;
+    // every ligand in its own form unless the context set a launch shape or form
+    b.cfg.ring = own_forms(c) && c->opts.threads_per_pose == 0 && c->opts.poses_per_block == 0;
     if (c->opts.threads_per_pose > 0) {   // the context's launch shape, until tuned
         b.cfg.tpp = c->opts.threads_per_pose;
         b.cfg.ppb = c->opts.poses_per_block > 0 ? c->opts.poses_per_block : 128 / b.cfg.tpp;
@@ -2050,7 +2083,7 @@ extern "C" int batch_local_search_dev(adgb_ctx *c, int batch_id, float *genes_de
     EvalCfg cfg = b.cfg;
     if (!b.tuned || p->reduce_variant >= 0) cfg.variant = variant;
     cfg.paired = cfg.paired && batch_pairable(b, cfg);
-    cfg.ring = cfg.ring && batch_ringable(b);
+    cfg.ring = cfg.ring && batch_has_large(b);
     cudaError_t e = cudaSuccess;
     const bool same = b.cur && b.k_genes == genes_dev && b.k_energy == best_energy_dev &&
                       b.k_iters == p->iters && b.k_rho == p->rho && b.k_eps == p->eps &&
@@ -2102,8 +2135,8 @@ extern "C" int batch_autotune(adgb_ctx *c, int batch_id, const float *genes_dev,
     if (iters < 1 || (b.total > 0 && !genes_dev)) return fail(c, ADGB_EINVAL, "batch_autotune: bad arguments");
     DeviceGuard g(c->device);
     // one genotype a warp (the last field 0); where every ligand of the batch
-    // qualifies, two genotypes a warp; where any has a ring table, the ring
-    // sweep for those and two genotypes a warp for the smaller ones
+    // qualifies, two genotypes a warp; where any has more than 32 atoms, every
+    // ligand in its own form (item_cfg)
     const EvalCfg all[] = {{32, 4, ADGB_REDUCE_SHFL, 1, 0, 0}, {32, 4, ADGB_REDUCE_MMA_TF32X2, 1, 0, 0},
                            {32, 4, ADGB_REDUCE_MMA_BF16X3, 1, 0, 0}, {32, 4, ADGB_REDUCE_TCGEN05, 1, 0, 0},
                            {32, 2, ADGB_REDUCE_SHFL, 1, 0, 0}, {64, 2, ADGB_REDUCE_SHFL, 1, 0, 0},
@@ -2112,8 +2145,8 @@ extern "C" int batch_autotune(adgb_ctx *c, int batch_id, const float *genes_dev,
                            {128, 2, ADGB_REDUCE_SHFL, 1, 0, 0, 1}, {128, 2, ADGB_REDUCE_TCGEN05, 1, 0, 0, 1}};
     std::vector<EvalCfg> cands;
     for (const EvalCfg &cf : all)
-        if (c->opts.genotypes_per_warp == 0 ? (!cf.paired || batch_pairable(b, cf)) && (!cf.ring || batch_ringable(b))
-                                            : !cf.paired && !cf.ring)
+        if ((!cf.paired || (c->opts.genotypes_per_warp == 0 && batch_pairable(b, cf))) &&
+            (!cf.ring || (own_forms(c) && batch_has_large(b))))
             cands.push_back(cf);
     const size_t gbytes = sizeof(float) * (size_t)b.total * (6 + ADGB_MAX_TORS);
     float *tg = nullptr, *te = nullptr;

@@ -167,3 +167,63 @@ def test_mixed_batch_equals_single_ligand_calls(pkg, rec, variant):
         assert np.array_equal(gb[at:at + len(g), :g.shape[1]], x), lid
         at += len(g)
     ctx.close()
+
+
+# about a tenth of the pairs listed; the last of a size is on the ring's side
+SPARSE = [(40, 1), (52, 1), (56, 1), (57, 1), (64, 2), (80, 1), (90, 1), (90, 2), (112, 1), (112, 2),
+          (128, 2), (128, 4), (129, 1), (160, 1), (200, 2), (256, 2)]
+
+
+def thinned(lig, share, seed=3):
+    """The ligand with a share of its pairs."""
+    k = max(1, int(share * len(lig["pairs"])))
+    keep = np.sort(np.random.default_rng(seed).permutation(len(lig["pairs"]))[:k])
+    return dict(lig, pairs=np.ascontiguousarray(lig["pairs"][keep]))
+
+
+@pytest.mark.parametrize("n_atoms, n_tors", SPARSE)
+def test_large_ligands_with_few_pairs_match_oracle(pkg, rec, n_atoms, n_tors):
+    """Few torsions list few of a large ligand's pairs: such ligands may leave
+    the ring for the other kernels, on either side of the line."""
+    lig = synth.make_ligand(50_000 + n_atoms, n_atoms, 4, n_tors)
+    genes = synth.make_poses(51_000 + n_atoms, 3, rec, lig["n_tors"])
+    genes[:, 6:] *= 0.05
+    R = oracle.Receptor(rec)
+    for l in (lig, thinned(lig, 0.1)):
+        ctx = pkg.Context(0)
+        rid, lid = check_scores(pkg, ctx, rec, l, genes, 0)
+        best, gb, _ = ctx.local_search(rid, lid, genes.copy(), 8)
+        L = oracle.Ligand(l)
+        for p in range(len(genes)):
+            er = oracle.score(R, L, gb[p])[0]
+            assert abs(best[p] - er) <= max(1e-4 * abs(er), 1e-3), (p, best[p], er)
+        ctx.close()
+
+
+def test_sparse_and_dense_ligands_share_a_batch(pkg, rec):
+    """Ligands of every form in one batch, each at sizes where its batch form
+    is its single call's: the single calls' bits."""
+    import torch
+    ligs = [synth.make_ligand(52_000 + a, a, 4, t) for a, t in
+            ((20, 4), (40, 8), (52, 1), (56, 1), (52, 12), (96, 1), (112, 1), (112, 20), (140, 30))]
+    ligs.append(thinned(synth.make_ligand(52_300, 200, 4, 8), 0.02))
+    genes = [synth.make_poses(52_400 + i, 3 + i, rec, l["n_tors"]) for i, l in enumerate(ligs)]
+    ctx = pkg.Context(0)
+    rid = ctx.upload_receptor_grids(rec)
+    lids = [ctx.upload_ligand_torsion_tree(l) for l in ligs]
+    bid = ctx.batch_create([rid] * len(ligs), lids, [len(g) for g in genes])
+    g0 = np.zeros((sum(len(g) for g in genes), 46), np.float32)
+    at = 0
+    for g in genes:
+        g0[at:at + len(g), :g.shape[1]] = g
+        at += len(g)
+    gd, ed = torch.from_numpy(g0).cuda(), torch.empty(len(g0), device="cuda")
+    ctx.batch_local_search_dev(bid, gd, ed, 15)
+    gb, eb = gd.cpu().numpy(), ed.cpu().numpy()
+    at = 0
+    for lid, g in zip(lids, genes):
+        b, x, _ = ctx.local_search(rid, lid, g.copy(), 15)
+        assert np.array_equal(eb[at:at + len(g)], b), lid
+        assert np.array_equal(gb[at:at + len(g), :g.shape[1]], x), lid
+        at += len(g)
+    ctx.close()
