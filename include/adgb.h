@@ -88,9 +88,10 @@ typedef struct {
                               arithmetic in packed FP32x2 instructions - a warp for ligands of
                               at most 32 atoms (with matching rounds, at most 26 torsions, one
                               warp a genotype's atoms), a block (ring sweep of the pairs) for
-                              larger ones that list enough of their pairs (about an eighth or
-                              more) where neither threads_per_pose nor poses_per_block nor
-                              pair_rounds asks for another form; 1: one genotype a warp or
+                              larger ones that list enough of their pairs (about a tenth of
+                              them up to 48 atoms, a quarter above) where neither
+                              threads_per_pose and poses_per_block (unless 128 and 2) nor
+                              pair_rounds ask for another form; 1: one genotype a warp or
                               group of warps */
 } adgb_options;
 
@@ -407,10 +408,11 @@ int rescore_fp64_dev(adgb_ctx *ctx, int receptor_id, int ligand_id, const float 
  * pair counts), each against its own receptor, locally searched by one
  * multi-ligand call.  Every kind of ligand the batch holds (up to 32 atoms;
  * larger ones by the ring sweep's 3, 4 or 5 atoms a lane, or with few pairs by
- * the threads of a genotype) is one launch over its work items (a few genotypes of one ligand, longest first), and the
- * launches run side by side, so big and small ligands share the GPU without
- * stragglers; a context with a launch shape of its own runs one persistent
- * launch over all items.  The launches are captured into a CUDA graph on the
+ * the threads of a genotype) is one launch over its work items (a few genotypes
+ * of one ligand, longest first), and the launches run side by side, so big and
+ * small ligands share the GPU without stragglers; a context with a launch shape
+ * of its own (other than 128 threads and 2 genotypes a block) runs one
+ * persistent launch over all items.  The launches are captured into a CUDA graph on the
  * first call and replayed by later calls with the same buffers and parameters.
  * A call with others may come while earlier ones still run (the third such
  * call in a row waits on the host for the first).
@@ -428,7 +430,8 @@ int rescore_fp64_dev(adgb_ctx *ctx, int receptor_id, int ligand_id, const float 
  *   own stream after the caller's work is complete; not modified), keeps the
  *   fastest for this batch and for later batches of the same size class
  *   (largest ligand in 32-atom and 512-pair steps), and writes it to chosen
- *   (may be NULL).  Synchronous.
+ *   (may be NULL).  A context created with the chosen shape and variant runs
+ *   such a batch the same way.  Synchronous.
  * batch_local_search_dev - local_search over every genotype of the batch:
  *   genes [total][ADGB_MAX_GENES] in/out, best_energy [total] out, on
  *   `stream`.  p->flags must not ask for resume.

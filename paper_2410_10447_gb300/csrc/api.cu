@@ -806,6 +806,12 @@ int build_ligand(std::string *err, const adgb_ligand_desc *d, HostLigand &h) {
 
 }  // namespace
 
+// Whether the launch shape options allow the ring sweep: none set, or its own
+// shape (batch_autotune reports it as such).
+static bool ring_shape_opts(int tpp, int ppb) {
+    return (tpp == 0 && ppb == 0) || (tpp == 32 * RING_WARPS && ppb == 2);
+}
+
 // The launch shape of a ligand (every single-ligand call, dock() and each
 // served job take it, so that they compute the same bits).
 EvalCfg adgb::launch_cfg(const LigDev &L, int tpp_opt, int ppb_opt, int variant,
@@ -834,9 +840,9 @@ EvalCfg adgb::launch_cfg(const LigDev &L, int tpp_opt, int ppb_opt, int variant,
     cfg.paired = genotypes_per_warp == 0 &&
                  pair_eligible(L.n_atoms, L.n_tors, L.n_pairs, L.n_rounds, L.r_lanes, cfg.tpp);
     // above 32 atoms the ring sweep, two genotypes a block, where the ligand has
-    // its table, unless the caller set a launch shape or asked for one genotype
-    // a warp
-    cfg.ring = genotypes_per_warp == 0 && tpp_opt == 0 && ppb_opt == 0 && L.ring_n > 0;
+    // its table, unless the caller set another launch shape or asked for one
+    // genotype a warp
+    cfg.ring = genotypes_per_warp == 0 && ring_shape_opts(tpp_opt, ppb_opt) && L.ring_n > 0;
     return cfg;
 }
 
@@ -2038,8 +2044,8 @@ extern "C" int batch_create(adgb_ctx *c, int n_items, const int *receptor_ids, c
     b.cfg.variant = c->opts.reduce_variant;
     b.cfg.paired = c->opts.genotypes_per_warp == 0;
     // every ligand in its own form unless the context set a launch shape or form
-    b.cfg.ring = own_forms(c) && c->opts.threads_per_pose == 0 && c->opts.poses_per_block == 0;
-    if (c->opts.threads_per_pose > 0) {   // the context's launch shape, until tuned
+    b.cfg.ring = own_forms(c) && ring_shape_opts(c->opts.threads_per_pose, c->opts.poses_per_block);
+    if (c->opts.threads_per_pose > 0 && !b.cfg.ring) {   // the context's launch shape, until tuned
         b.cfg.tpp = c->opts.threads_per_pose;
         b.cfg.ppb = c->opts.poses_per_block > 0 ? c->opts.poses_per_block : 128 / b.cfg.tpp;
     }

@@ -196,3 +196,35 @@ def test_batch_of_small_ligands_searches_every_genotype(pkg, torch, ppb, variant
         assert np.array_equal(g.cpu().numpy()[r:r + len(x), :x.shape[1]], y)
         r += len(x)
     ctx.close()
+
+
+def test_context_of_the_autotuned_shape_runs_the_batch_the_same_way(pkg, torch):
+    """Large ligands, whose fastest form (two genotypes a 128-thread block) is
+    no launch shape of one genotype's threads; the context takes small ones too."""
+    rec = synth.make_receptor(synth.generate.BASE_SEED + 6, 48, 6)
+    ligs = [synth.make_ligand(900 + a, a, 6, 16) for a in (72, 90)]
+    small = synth.make_ligand(901, 20, 6, 4)
+    n = 300
+    starts = torch.from_numpy(pack([synth.make_poses(910 + i, n, rec, 16) for i in range(2)])).cuda()
+
+    def search(ctx, tune):
+        rid = ctx.upload_receptor_grids(rec)
+        bid = ctx.batch_create([rid] * 2, [ctx.upload_ligand_torsion_tree(L) for L in ligs], [n] * 2)
+        chosen = ctx.batch_autotune(bid, starts, iters=10) if tune else None
+        g, e = starts.clone(), torch.empty(2 * n, device="cuda")
+        ctx.batch_local_search_dev(bid, g, e, 10)
+        return g.cpu().numpy(), e.cpu().numpy(), chosen
+
+    ctx = pkg.Context(0)
+    g, e, chosen = search(ctx, True)
+    assert (chosen["threads_per_pose"], chosen["poses_per_block"]) == (128, 2)
+    again = pkg.Context(0, **chosen)
+    g2, e2, _ = search(again, False)
+    assert np.array_equal(g, g2) and np.array_equal(e, e2)
+    rid, lid = again.upload_receptor_grids(rec), again.upload_ligand_torsion_tree(small)
+    x = torch.from_numpy(pack([synth.make_poses(920, 5, rec, 4)])).cuda()
+    es = torch.full((5,), float("nan"), device="cuda")
+    again.batch_local_search_dev(again.batch_create([rid], [lid], [5]), x, es, 10)
+    assert np.all(np.isfinite(es.cpu().numpy()))
+    ctx.close()
+    again.close()
