@@ -151,3 +151,23 @@ def test_sw_whole_searches(pkg, torch, cfg1):
         with pytest.raises(pkg.AdgbError):
             ctx.local_search_sw(rid, lid, g0[:2], pkg.adgb.sw_params(**bad))
     ctx.close()
+
+
+@pytest.mark.parametrize("n_atoms, n_tors", [(16, 4), (32, 8), (45, 11), (64, 12), (90, 20), (200, 30)])
+def test_sw_bits_do_not_depend_on_the_launch_size(pkg, torch, n_atoms, n_tors):
+    """Launches of few blocks an SM run a kernel with more registers: a
+    genotype's search takes the same decisions, to the bit, in each (pair
+    list and matching rounds, one, two and four warps a genotype)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    rec = synth.make_receptor(synth.generate.BASE_SEED + 8, 48, 4)
+    lig = synth.make_ligand(3000 + n_atoms, n_atoms, 4, n_tors)
+    many = 2 * sms * 4 + 9          # above two blocks an SM at four genotypes a block
+    genes = np.tile(synth.make_poses(3001, 24, rec, n_tors), (many // 24 + 1, 1))[:many]
+    ctx = pkg.Context(0)
+    rid, lid = ctx.upload_receptor_grids(rec), ctx.upload_ligand_torsion_tree(lig)
+    p = pkg.adgb.sw_params(max_evals=80, rho0=0.5, seed=12)
+    e, g, ev, st = ctx.local_search_sw(rid, lid, genes[:24].copy(), p, want_state=True)
+    e2, g2, ev2, st2 = ctx.local_search_sw(rid, lid, genes.copy(), p, want_state=True)
+    assert np.array_equal(ev, ev2[:24]) and np.array_equal(e, e2[:24])
+    assert np.array_equal(g, g2[:24]) and np.array_equal(st, st2[:24])
+    ctx.close()
