@@ -550,10 +550,12 @@ __device__ __forceinline__ void search_ring(unsigned char *sm, const RingSmem &L
 // 300 genotypes, one block an SM: 45 atoms 70 -> 73 -> 74, 90 36 -> 40 -> 41,
 // 160 16 -> 18 -> 22, 256 7.0 -> 9.0 -> 10.7; 900 genotypes, three, 4 -> 3: 45
 // atoms 160 -> 166, 160 32 -> 34).  Larger launches: 5 for a = 3 up to 96 atoms
-// (12 000 genotypes of 45 atoms 206 -> 214, of 90 atoms 91.8 -> 92.4), 3 from
-// 250 atoms on, where a fourth block's shared memory does not fit (256 atoms,
-// 40 torsions, 8192 genotypes 15.9 -> 17.7) or leaves the L1 cache little (256
-// atoms, 20 torsions, 4000 genotypes 15.8 -> 16.7), else 4 (128 atoms, 8000
+// (12 000 genotypes of 45 atoms 206 -> 214, of 90 atoms 91.8 -> 92.4), 3 above
+// 192 atoms (four atoms a lane over two windows, the most registers a thread:
+// times with 4 blocks over those with 3 for 4000 and 8192 genotypes, 64^3 grid
+// 1.01 at 193 atoms, 1.02 at 220, 1.03 at 240 and 256, 128^3 grid 1.00-1.02,
+// 1.05, 1.07, 1.08; 1500 genotypes 1.12-1.20), else 4 (161 to 192 atoms, as much
+// shared memory a block but three atoms a lane: 0.95-0.97; 128 atoms, 8000
 // genotypes, 3 -> 4: 52.5 -> 53.2).  Four blocks an SM that do not fit also run
 // as 3 (256 atoms, 40 torsions, 1000 genotypes 10.6 -> 12.5).
 template <int A, int VAR, int MB>
@@ -643,7 +645,7 @@ cudaError_t launch_ring_mb(const RingArgs &a, int need, int fit, int threads, in
                            cudaStream_t s) {
     if constexpr (VAR == ADGB_REDUCE_SHFL) {
         if (need <= 2) return launch_ring_t<A, VAR, 2>(a, threads, smem, s);
-        if (need <= 3 || fit <= 3 || (need > 4 && a.lig.n_atoms >= 250))
+        if (need <= 3 || fit <= 3 || (A == 4 && need > 4 && a.L.r.windows > 1))
             return launch_ring_t<A, VAR, 3>(a, threads, smem, s);
     }
     if constexpr (A == 3)

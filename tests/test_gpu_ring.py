@@ -227,3 +227,10 @@ def test_sparse_and_dense_ligands_share_a_batch(pkg, rec):
         assert np.array_equal(gb[at:at + len(g), :g.shape[1]], x), lid
         at += len(g)
     ctx.close()
+
+
+@pytest.mark.parametrize("n_atoms", [161, 176, 193, 220])
+def test_ring_bits_of_two_windows_do_not_depend_on_the_launch_size(pkg, rec, n_atoms):
+    """Three and four atoms a lane over two windows of lanes: another number
+    of blocks an SM in large launches on either side of 192 atoms."""
+    test_ring_bits_do_not_depend_on_the_launch_size(pkg, rec, n_atoms)
