@@ -245,8 +245,10 @@ struct RingShape {
                           // step), and copies: one a team, or one a warp with windows
     int pos_res, copy_res; // a = 4: entries a residue class (ring_index)
 };
-// a = 3, 4 or 5, whichever leaves the fewest idle lanes at N atoms (256 atoms:
-// 64 lanes of 4; with 3 a lane 86 of 96 lanes, with 5 52 of 64).
+// a = 3, 4 or 5 by the atoms: over each range about the fewest idle lanes (256
+// atoms: 64 lanes of 4; with 3 a lane 86 of 96 lanes, with 5 52 of 64), not at
+// each of its sizes (at 33-40 atoms 4 a lane would leave 2-5 idle instead of
+// 4-10, at 49 and 50 5 a lane 2 instead of 6, in tables 11 and 6% smaller).
 __host__ __device__ inline RingShape ring_shape(int N) {
     RingShape r;
     r.a = N <= 48 ? 3 : N <= 64 ? 4 : N <= 80 ? 5 : N <= 96 ? 3 : N <= 128 ? 4 : N <= 160 ? 5

@@ -1,8 +1,8 @@
-// Fused scoring / ADADELTA local search of ligands of more than 32 atoms
-// (Sec. 2.1, Sec. 3; Table 1's gpu_gradient_minAD): one block of 4 warps
-// searches two genotypes, packed (genotype A in .x, B in .y), so that
-// the ligand's pair constants, torsion tree and addresses are read and
-// computed once for both.
+// Fused scoring / ADADELTA local search of ligands of more than 32 atoms that
+// list enough of their pairs (Sec. 2.1, Sec. 3; Table 1's gpu_gradient_minAD):
+// one block of 4 warps searches two genotypes, packed (genotype A in .x, B in
+// .y), so that the ligand's pair constants, torsion tree and addresses are read
+// and computed once for both.
 //
 // The intramolecular pairs are swept as a ring (RingShape): a lane holds A
 // consecutive atoms of both genotypes in registers, and at step s meets atom
@@ -10,24 +10,24 @@
 // lane's j is another atom, so the reaction on j is added to the warp's own
 // copy of the forces in shared memory without atomics: two loads, two stores
 // and a warp barrier for A pairs of two genotypes, all of them free of bank
-// conflicts (ring_index).  The steps
-// are split over the block's warps (and, for small ligands, over two or three
-// teams of lanes in a warp); every atom's owner then sums the copies.  The
-// pair constants come from a table in the order of the sweep (coalesced
-// 16-byte loads), zeros for pairs that are not listed, the H-bond flag in the
-// sign of A.
+// conflicts (ring_index).  The steps are split over the block's warps (and, for
+// small ligands, over two teams of lanes in a warp); every atom's owner then
+// sums the copies.  The pair constants come from a table in the order of the
+// sweep (coalesced 16-byte loads), zeros for pairs that are not listed, the
+// H-bond flag in the sign of A.
 //
 // What bounds it: from ~90 atoms on, the issue and FMA pipe of the pair terms
 // (26 packed and 14 scalar instructions for a pair of two genotypes, 15 more
 // for distances, sums and the reaction; 256 atoms: FMA pipe 52%, issue 47%,
 // LSU data pipe 37% busy, the rest fixed latencies at 10-15 warps an SM); below
-// that, the latency of an evaluation's six barriers, gene threads, torsion walk
+// that, the latency of an evaluation's five barriers, gene threads, torsion walk
 // and grid loads (45 atoms, one block an SM: ring 2300 of 6500 cycles, gene
-// threads 1000, walk 700, grid 700, torsions 950, atoms' sums 650).  The kernel it took over from for these ligands (one genotype a 64-
-// or 128-thread group, forces through per-pair slots in shared memory) had its
-// LSU data pipe 73% busy at 256 atoms, 46% of the shared-memory wavefronts
-// bank-conflict replays, at 107K warp instructions an evaluation; this one
-// issues 40K.  Local search, M evaluations/s before -> with the sweep:
+// threads 1000, walk 700, grid 700, torsions 950, atoms' sums 650).  The kernel
+// it took over from for these ligands (one genotype a 64- or 128-thread group,
+// forces through per-pair slots in shared memory) had its LSU data pipe 73%
+// busy at 256 atoms, 46% of the shared-memory wavefronts bank-conflict replays,
+// at 107K warp instructions an evaluation; this one issues 40K.  Local search,
+// M evaluations/s before -> with the sweep:
 // 45 atoms x 1000 genotypes 95 -> 157, 64 x 8000 58 -> 121, 90 x 1500
 // 31 -> 87, 128 x 8000 17 -> 53, 160 x 6000 12 -> 38, 256 x 2048 6.2 -> 16.0
 // (with 3 or 5 atoms a lane only, no 4, and then 4: 64 x 8000 113 -> 121, 128 x
