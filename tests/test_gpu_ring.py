@@ -169,7 +169,7 @@ def test_mixed_batch_equals_single_ligand_calls(pkg, rec, variant):
     ctx.close()
 
 
-# about a tenth of the pairs listed; the last of a size is on the ring's side
+# one or two torsions: on either side of the line (thinned, all off the ring)
 SPARSE = [(40, 1), (52, 1), (56, 1), (57, 1), (64, 2), (80, 1), (90, 1), (90, 2), (112, 1), (112, 2),
           (128, 2), (128, 4), (129, 1), (160, 1), (200, 2), (256, 2)]
 
